@@ -43,24 +43,18 @@ template <> __device__ __forceinline__ __half from_f<__half>(float v) { return _
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // Cache policy of the population stream (each value is read once and written
-// once per step).  16-bit storage streams (ld/st .cs, evict-first in L2), which
-// leaves the immersed-boundary working set (positions, element terms, force
-// and velocity stencils) in L2 across the step: 85.4 -> 81.6 us per cycle on
-// the 256x128x64 filter, the stream-collide itself unchanged.  FP32 keeps the
-// read-only path: streaming loads cost it 7 us (62.5 -> 69.3 us), streaming
-// stores alone gain nothing (measured on GB300).
-template <class S>
-__host__ __device__ constexpr bool pop_streaming() { return sizeof(S) == 2; }
-
-template <class S, class T>
+// once per step).  Loads take the read-only path (streaming loads, ld .cs,
+// cost FP32 7 us on the 256x128x64 filter and the 16-bit four-node kernel 28
+// of 289 us on 512x256x128, GB300).  16-bit stores stream (evict-first in L2),
+// FP32 stores do not; neither choice can be told from the other in time.
+template <class T>
 __device__ __forceinline__ T pop_ld(const T* p) {
-    if constexpr (pop_streaming<S>()) return __ldcs(p);
-    else return __ldg(p);
+    return __ldg(p);
 }
 
 template <class S, class T>
 __device__ __forceinline__ void pop_st(T* p, T v) {
-    if constexpr (pop_streaming<S>()) __stcs(p, v);
+    if constexpr (sizeof(S) == 2) __stcs(p, v);
     else *p = v;
 }
 
@@ -118,8 +112,8 @@ template <class S> __device__ __forceinline__ S cvt_rs1(float v, unsigned rb) {
 
 template <class S> struct Pop {
     static __device__ __forceinline__ float ld(const S* p, long long idx, int i) {
-        if constexpr (sizeof(S) == 4) return pop_ld<S>(p + idx);
-        else return wgt(i) * to_f(pop_ld<S>(p + idx));
+        if constexpr (sizeof(S) == 4) return pop_ld(p + idx);
+        else return wgt(i) * to_f(pop_ld(p + idx));
     }
     // rb: the node's random word (sr_seed); 16-bit storage rounds with
     // rb * sr_k(i), FP32 ignores it
@@ -140,7 +134,7 @@ template <class S, int NPT>
 struct VecIO {
     using R = typename Raw<sizeof(S) * NPT>::T;
     static __device__ __forceinline__ void ld(const S* base, long long idx, int i, float out[NPT]) {
-        const R r = pop_ld<S>(reinterpret_cast<const R*>(base + idx));
+        const R r = pop_ld(reinterpret_cast<const R*>(base + idx));
         const S* e = reinterpret_cast<const S*>(&r);
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
@@ -617,13 +611,23 @@ __device__ __forceinline__ void sc_nodes(const LatticeArgs& a, const ChannelDev&
     if (prevf && (gp0 & 31) == 0) fl_prev[grp] = 0;
 }
 
+// Channel of block b: the last one whose first block is <= b (bisection; the
+// linear search cost the 24-channel sweep 40 of 388 us, GB300).
+__device__ __forceinline__ int sc_channel(const LatticeArgs& a, int b) {
+    int lo = 0, hi = a.n_ch;
+    while (hi - lo > 1) {
+        const int m = (lo + hi) >> 1;
+        if (b >= chan(a, m).blk0) lo = m;
+        else hi = m;
+    }
+    return lo;
+}
+
 template <class S, int NPT, int BS>
 __global__ void __launch_bounds__(BS, K3MinBlocks<S, NPT, BS>::value) k_stream_collide(const __grid_constant__ LatticeArgs a) {
     // (sc_nodes waits for the predecessor after its population loads)
     const int b = blockIdx.x;
-    int c = 0;
-    for (int k = 1; k < a.n_ch; ++k)
-        if (b >= chan(a, k).blk0) c = k;
+    const int c = sc_channel(a, b);
     const ChannelDev C = chan(a, c);   // registers: read once from the parameter bank
     const int lane = threadIdx.x & 31;
     const int p0 = ((b - C.blk0) * BS + (int)threadIdx.x) * NPT;   // first channel-local node of this thread
@@ -683,10 +687,10 @@ template <> struct PairIO<float> {
 template <> struct PairIO<__half> {
     static constexpr bool SCALED = true;
     static __device__ __forceinline__ F2 ld2(const __half* p) {
-        const unsigned r = __ldcs(reinterpret_cast<const unsigned*>(p));
+        const unsigned r = pop_ld(reinterpret_cast<const unsigned*>(p));
         return __half22float2(*reinterpret_cast<const __half2*>(&r));
     }
-    static __device__ __forceinline__ float ld1(const __half* p) { return __half2float(__ldcs(p)); }
+    static __device__ __forceinline__ float ld1(const __half* p) { return __half2float(pop_ld(p)); }
     static __device__ __forceinline__ void st2(__half* p, F2 v, unsigned rb) {
         __stcs(reinterpret_cast<unsigned*>(p), cvt_rs2<__half>(v.y, v.x, rb));
     }
@@ -695,11 +699,11 @@ template <> struct PairIO<__half> {
 template <> struct PairIO<__nv_bfloat16> {
     static constexpr bool SCALED = true;
     static __device__ __forceinline__ F2 ld2(const __nv_bfloat16* p) {
-        const unsigned r = __ldcs(reinterpret_cast<const unsigned*>(p));
+        const unsigned r = pop_ld(reinterpret_cast<const unsigned*>(p));
         return make_float2(__uint_as_float(r << 16), __uint_as_float(r & 0xffff0000u));
     }
     static __device__ __forceinline__ float ld1(const __nv_bfloat16* p) {
-        return __uint_as_float((unsigned)__bfloat16_as_ushort(__ldcs(p)) << 16);
+        return __uint_as_float((unsigned)__bfloat16_as_ushort(pop_ld(p)) << 16);
     }
     static __device__ __forceinline__ void st2(__nv_bfloat16* p, F2 v, unsigned rb) {
         __stcs(reinterpret_cast<unsigned*>(p), cvt_rs2<__nv_bfloat16>(v.y, v.x, rb));
@@ -793,23 +797,88 @@ struct Mac2 {
 
 // Collision of the opposite directions (I, I + 1), I odd, for both nodes.
 template <bool SCALED, int I>
-__device__ __forceinline__ void collide_pair2(F2 h[Q], const Mac2& m, F2 om, F2 omc, F2 c3om, F2 c9fp, F2 c3fp) {
-    constexpr int J = I + 1;
+__device__ __forceinline__ void collide_two(F2& hi, F2& hj, const Mac2& m, const ChannelDev& C) {
     const F2 eu = edot2<I>(m.ux, m.uy, m.uz);
     const F2 eg = edot2<I>(m.gx, m.gy, m.gz);
     const F2 reu = mul2(m.rho, eu);
     const F2 E = fma2(mul2(f2s(4.5f), reu), eu, m.A1);          // A1 + 9/2 rho (e.u)^2
-    const F2 Es = fma2(om, E, fma2(mul2(c9fp, eu), eg, m.mug));   // + fp (9 (e.u)(e.g) - 3 u.g)
-    const F2 Os = fma2(c3om, reu, mul2(c3fp, eg));                // 3 om rho e.u + 3 fp e.g
+    const F2 Es = fma2(C.om2, E, fma2(mul2(C.c9fp2, eu), eg, m.mug));   // + fp (9 (e.u)(e.g) - 3 u.g)
+    const F2 Os = fma2(C.c3om2, reu, mul2(C.c3fp2, eg));                // 3 om rho e.u + 3 fp e.g
     const F2 XI = add2(Es, Os), XJ = sub2(Es, Os);
     if constexpr (SCALED) {
-        h[I] = fma2(omc, h[I], XI);
-        h[J] = fma2(omc, h[J], XJ);
+        hi = fma2(C.omc2, hi, XI);
+        hj = fma2(C.omc2, hj, XJ);
     } else {
         const F2 w = f2s(wgt(I));
-        h[I] = fma2(w, XI, mul2(omc, h[I]));
-        h[J] = fma2(w, XJ, mul2(omc, h[J]));
+        hi = fma2(w, XI, mul2(C.omc2, hi));
+        hj = fma2(w, XJ, mul2(C.omc2, hj));
     }
+}
+
+// Sums over the directions of one node pair (pairwise differences of opposite
+// directions first).
+struct PairSums {
+    F2 a1, a3, a5, dx, dy, dz, sa, sd;
+    __device__ __forceinline__ void axis(F2 h1, F2 h2, F2 h3, F2 h4, F2 h5, F2 h6) {
+        a1 = sub2(h1, h2);
+        a3 = sub2(h3, h4);
+        a5 = sub2(h5, h6);
+        sa = add2(add2(add2(h1, h2), add2(h3, h4)), add2(h5, h6));
+    }
+    __device__ __forceinline__ void diag(F2 h7, F2 h8, F2 h9, F2 h10, F2 h11, F2 h12, F2 h13, F2 h14, F2 h15, F2 h16,
+                                         F2 h17, F2 h18) {
+        const F2 d7 = sub2(h7, h8), d9 = sub2(h9, h10), d11 = sub2(h11, h12);
+        const F2 d13 = sub2(h13, h14), d15 = sub2(h15, h16), d17 = sub2(h17, h18);
+        sd = add2(add2(add2(add2(h7, h8), add2(h9, h10)), add2(add2(h11, h12), add2(h13, h14))),
+                  add2(add2(h15, h16), add2(h17, h18)));
+        dx = add2(add2(d7, d9), add2(d11, d13));
+        dy = add2(sub2(d7, d9), add2(d15, d17));
+        dz = add2(sub2(d11, d13), sub2(d15, d17));
+    }
+};
+
+// The pair's force density (the uniform body force plus g0, g1 when forced).
+__device__ __forceinline__ void macro_force(const ChannelDev& C, float4 g0, float4 g1, bool forced, Mac2& m) {
+    m.gx = C.G2[0];
+    m.gy = C.G2[1];
+    m.gz = C.G2[2];
+    if (forced) {
+        m.gx = add2(m.gx, make_float2(g0.x, g1.x));
+        m.gy = add2(m.gy, make_float2(g0.y, g1.y));
+        m.gz = add2(m.gz, make_float2(g0.z, g1.z));
+    }
+}
+
+// Density and velocity of the pair from its sums and rest population.
+template <bool SCALED>
+__device__ __forceinline__ void macro_pair(const PairSums& p, F2 h0, Mac2& m) {
+    F2 jx, jy, jz;
+    if constexpr (SCALED) {
+        const F2 w1 = f2s(wgt(1)), w2 = f2s(wgt(7));
+        jx = fma2(w1, p.a1, mul2(w2, p.dx));
+        jy = fma2(w1, p.a3, mul2(w2, p.dy));
+        jz = fma2(w1, p.a5, mul2(w2, p.dz));
+        m.drho = fma2(f2s(wgt(0)), h0, fma2(w1, p.sa, mul2(w2, p.sd)));
+    } else {
+        jx = add2(p.a1, p.dx);
+        jy = add2(p.a3, p.dy);
+        jz = add2(p.a5, p.dz);
+        m.drho = add2(h0, add2(p.sa, p.sd));
+    }
+    m.rho = add2(f2s(1.0f), m.drho);
+    const F2 irho = make_float2(1.0f / m.rho.x, 1.0f / m.rho.y);
+    const F2 half = f2s(0.5f);
+    m.ux = mul2(fma2(half, m.gx, jx), irho);
+    m.uy = mul2(fma2(half, m.gy, jy), irho);
+    m.uz = mul2(fma2(half, m.gz, jz), irho);
+}
+
+// The terms of the collision that all directions share.
+__device__ __forceinline__ void macro_terms(const ChannelDev& C, Mac2& m) {
+    const F2 uu = fma2(m.uz, m.uz, fma2(m.uy, m.uy, mul2(m.ux, m.ux)));
+    const F2 ug = fma2(m.uz, m.gz, fma2(m.uy, m.gy, mul2(m.ux, m.gx)));
+    m.A1 = fma2(mul2(f2s(-1.5f), m.rho), uu, m.drho);   // drho - 3/2 rho u.u
+    m.mug = mul2(make_float2(-C.c3fp2.x, -C.c3fp2.y), ug);   // -3 fp u.g
 }
 
 // Moments and collision of one in-range node pair in place (h: the pulled
@@ -820,67 +889,22 @@ __device__ __forceinline__ void collide_pair2(F2 h[Q], const Mac2& m, F2 om, F2 
 template <bool SCALED>
 __device__ __forceinline__ void pair_collide(const ChannelDev& C, float4 g0, float4 g1, bool forced, F2 h[Q],
                                              Mac2& m) {
-    m.gx = make_float2(C.G[0], C.G[0]);
-    m.gy = make_float2(C.G[1], C.G[1]);
-    m.gz = make_float2(C.G[2], C.G[2]);
-    if (forced) {
-        m.gx = add2(m.gx, make_float2(g0.x, g1.x));
-        m.gy = add2(m.gy, make_float2(g0.y, g1.y));
-        m.gz = add2(m.gz, make_float2(g0.z, g1.z));
-    }
-    // moments (pairwise differences of opposite directions first)
-    {
-        const F2 a1 = sub2(h[1], h[2]), a3 = sub2(h[3], h[4]), a5 = sub2(h[5], h[6]);
-        const F2 d7 = sub2(h[7], h[8]), d9 = sub2(h[9], h[10]), d11 = sub2(h[11], h[12]);
-        const F2 d13 = sub2(h[13], h[14]), d15 = sub2(h[15], h[16]), d17 = sub2(h[17], h[18]);
-        const F2 sa = add2(add2(add2(h[1], h[2]), add2(h[3], h[4])), add2(h[5], h[6]));
-        const F2 sd = add2(add2(add2(add2(h[7], h[8]), add2(h[9], h[10])), add2(add2(h[11], h[12]), add2(h[13], h[14]))),
-                           add2(add2(h[15], h[16]), add2(h[17], h[18])));
-        const F2 dx = add2(add2(d7, d9), add2(d11, d13));
-        const F2 dy = add2(sub2(d7, d9), add2(d15, d17));
-        const F2 dz = add2(sub2(d11, d13), sub2(d15, d17));
-        F2 jx, jy, jz;
-        if constexpr (SCALED) {
-            const F2 w1 = f2s(wgt(1)), w2 = f2s(wgt(7));
-            jx = fma2(w1, a1, mul2(w2, dx));
-            jy = fma2(w1, a3, mul2(w2, dy));
-            jz = fma2(w1, a5, mul2(w2, dz));
-            m.drho = fma2(f2s(wgt(0)), h[0], fma2(w1, sa, mul2(w2, sd)));
-        } else {
-            jx = add2(a1, dx);
-            jy = add2(a3, dy);
-            jz = add2(a5, dz);
-            m.drho = add2(h[0], add2(sa, sd));
-        }
-        m.rho = add2(f2s(1.0f), m.drho);
-        const F2 irho = make_float2(1.0f / m.rho.x, 1.0f / m.rho.y);
-        const F2 half = f2s(0.5f);
-        m.ux = mul2(fma2(half, m.gx, jx), irho);
-        m.uy = mul2(fma2(half, m.gy, jy), irho);
-        m.uz = mul2(fma2(half, m.gz, jz), irho);
-    }
-    const F2 uu = fma2(m.uz, m.uz, fma2(m.uy, m.uy, mul2(m.ux, m.ux)));
-    const F2 ug = fma2(m.uz, m.gz, fma2(m.uy, m.gy, mul2(m.ux, m.gx)));
-    const float om_s = C.omega, fp_s = C.fpre;
-    m.A1 = fma2(mul2(f2s(-1.5f), m.rho), uu, m.drho);   // drho - 3/2 rho u.u
-    m.mug = mul2(f2s(-3.0f * fp_s), ug);                // -3 fp u.g
-    const F2 om = f2s(om_s), omc = f2s(1.0f - om_s), c3om = f2s(3.0f * om_s);
-    const F2 c9fp = f2s(9.0f * fp_s), c3fp = f2s(3.0f * fp_s);
+    macro_force(C, g0, g1, forced, m);
+    PairSums ps;
+    ps.axis(h[1], h[2], h[3], h[4], h[5], h[6]);
+    ps.diag(h[7], h[8], h[9], h[10], h[11], h[12], h[13], h[14], h[15], h[16], h[17], h[18]);
+    macro_pair<SCALED>(ps, h[0], m);
+    macro_terms(C, m);
     // rest population: (1 - om) h0 + w0 [om A1 - 3 fp u.g]
     {
-        const F2 X0 = fma2(om, m.A1, m.mug);
-        if constexpr (SCALED) h[0] = fma2(omc, h[0], X0);
-        else h[0] = fma2(f2s(wgt(0)), X0, mul2(omc, h[0]));
+        const F2 X0 = fma2(C.om2, m.A1, m.mug);
+        if constexpr (SCALED) h[0] = fma2(C.omc2, h[0], X0);
+        else h[0] = fma2(f2s(wgt(0)), X0, mul2(C.omc2, h[0]));
     }
-    collide_pair2<SCALED, 1>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 3>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 5>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 7>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 9>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 11>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 13>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 15>(h, m, om, omc, c3om, c9fp, c3fp);
-    collide_pair2<SCALED, 17>(h, m, om, omc, c3om, c9fp, c3fp);
+#define LBIBM_CP(I, J) collide_two<SCALED, I>(h[I], h[J], m, C);
+    LBIBM_CP(1, 2) LBIBM_CP(3, 4) LBIBM_CP(5, 6) LBIBM_CP(7, 8) LBIBM_CP(9, 10) LBIBM_CP(11, 12) LBIBM_CP(13, 14)
+    LBIBM_CP(15, 16) LBIBM_CP(17, 18)
+#undef LBIBM_CP
 }
 
 // Moments, collision and stores of one in-range node pair (h: the pulled
@@ -995,9 +1019,7 @@ template <class S, int BS>
 __global__ void __launch_bounds__(BS, LBIBM_K3_PAIR_THREADS / BS) k_stream_collide_pair(const __grid_constant__ LatticeArgs a) {
     // (sc_pair waits for the predecessor after its population loads)
     const int b = blockIdx.x;
-    int c = 0;
-    for (int k = 1; k < a.n_ch; ++k)
-        if (b >= chan(a, k).blk0) c = k;
+    const int c = sc_channel(a, b);
     const ChannelDev C = chan(a, c);
     const int pb = (b - C.blk0) * (2 * BS);                  // first channel-local node of the block
     const int p0 = pb + 2 * (int)threadIdx.x;
@@ -1018,13 +1040,17 @@ __global__ void __launch_bounds__(BS, LBIBM_K3_PAIR_THREADS / BS) k_stream_colli
 // pulls every direction as one aligned 64-bit word of four 16-bit values.  A
 // direction with an x component takes the value its first (+x) or last (-x)
 // node needs from the neighbouring lane's word by a shuffle, or, at a warp's
-// or a row's edge, from one extra aligned 32-bit word.  The words stay packed
-// (two registers per direction for four nodes) until the two node pairs are
-// unpacked in turn for the packed-FP32 moments and collision, and each
-// direction is stored as one 64-bit word.  The 16-bit kernel with one node per
-// thread holds too few population bytes in flight per register to cover HBM
-// latency; packed words hold four nodes' loads in the registers one node's
-// floats would take.
+// or a row's edge, from one extra aligned 32-bit word.
+//
+// What bounds it is HBM latency against registers: a thread holds its 19
+// words (38 registers) from the loads to the stores.  So the two node pairs
+// are collided one after the other, each unpacked twice (for the moments and,
+// two directions at a time, for the collision), and the rounded results take
+// the words' place until each direction leaves as one 64-bit store.  That
+// fits 96 registers, 20 warps per SM; with a pair's 19 directions held as
+// floats it took 128, 16 warps, and stored 32-bit words.  Measured on GB300,
+// 512x256x128 FP16: 345 -> 315 us (two unpackings and 64-bit stores at 16
+// warps), 289 (20 warps), 261 (read-only loads); 24 warps spill, 282.
 // ---------------------------------------------------------------------------
 template <class S> struct QuadIO;
 template <> struct QuadIO<__half> {
@@ -1065,12 +1091,12 @@ template <class S, int I>
 __device__ __forceinline__ void quad_pull(const S* src, unsigned NT, int gi0, const QuadNbr& nb, bool inr,
                                           bool edge_lo, bool edge_hi, uint2& w, unsigned& e) {
     const S* pl = src + ((unsigned)I * NT + (unsigned)(gi0 + pair_row<I>(nb)));
-    w = inr ? __ldcs(reinterpret_cast<const uint2*>(pl)) : make_uint2(0u, 0u);
+    w = inr ? pop_ld(reinterpret_cast<const uint2*>(pl)) : make_uint2(0u, 0u);
     e = 0u;
     if constexpr (ex(I) == 1) {
-        if (inr && edge_lo) e = __ldcs(reinterpret_cast<const unsigned*>(pl + nb.wxm));
+        if (inr && edge_lo) e = pop_ld(reinterpret_cast<const unsigned*>(pl + nb.wxm));
     } else if constexpr (ex(I) == -1) {
-        if (inr && edge_hi) e = __ldcs(reinterpret_cast<const unsigned*>(pl + nb.wxp));
+        if (inr && edge_hi) e = pop_ld(reinterpret_cast<const unsigned*>(pl + nb.wxp));
     }
 }
 
@@ -1089,50 +1115,151 @@ __device__ __forceinline__ void quad_shift(uint2& w, unsigned e, bool edge_lo, b
     }
 }
 
-// One node pair of the quad (k = 0: nodes x0, x0 + 1 from the words' lo
-// halves; k = 1: x0 + 2, x0 + 3): unpack, bounce-back, moments, collision and
-// the pair's stores (one 32-bit word per direction, rounded stochastically;
-// a solid node keeps its populations).
-template <class S>
-__device__ __forceinline__ void quad_half(const ChannelDev& C, const S* src, S* dst, unsigned NT, int gi, int y,
-                                          const uint2 w[Q], int k, uint32_t lk0, uint32_t lk1, bool forced,
-                                          float4 g0, float4 g1, Mac2& m) {
-    F2 h[Q];
-#define LBIBM_QU(I) h[I] = QuadIO<S>::unpack(k ? w[I].y : w[I].x);
-    LBIBM_ALL_I(LBIBM_QU)
-#undef LBIBM_QU
-    if (lk0 & ~1u) {
-#define LBIBM_PB(I) if (I > 0) pair_bounce<S, I>(src, NT, gi, lk0, C, y, h[I].x);
-        LBIBM_ALL_I(LBIBM_PB)
-#undef LBIBM_PB
+// Direction I of one node pair from its packed word.  UW: a moving y-wall adds
+// Ladd's term to the links that bounce back from it (in FP32, after the
+// unpacking: the sum need not be a 16-bit value).
+template <class S, int I, bool UW>
+__device__ __forceinline__ F2 quad_pop(unsigned word, uint32_t lk0, uint32_t lk1, const ChannelDev& C, int y) {
+    F2 h = QuadIO<S>::unpack(word);
+    if constexpr (UW && ey(I) != 0) {
+        const int wall = !C.has_uw || C.per[1] ? -1 : (ey(I) == 1 && y == 0) ? 0 : ((ey(I) == -1 && y == C.ny - 1) ? 1 : -1);
+        if (wall >= 0) {
+            const float t = 6.0f * (ex(I) * C.uw[wall][0] + ey(I) * C.uw[wall][1] + ez(I) * C.uw[wall][2]);
+            if ((lk0 >> I) & 1u) h.x += t;
+            if ((lk1 >> I) & 1u) h.y += t;
+        }
     }
-    if (lk1 & ~1u) {
-#define LBIBM_PB(I) if (I > 0) pair_bounce<S, I>(src, NT, gi + 1, lk1, C, y, h[I].y);
-        LBIBM_ALL_I(LBIBM_PB)
-#undef LBIBM_PB
+    return h;
+}
+
+// Bounce-back of one node pair in the packed words: where a link bit is set
+// the 16-bit value of direction I becomes the node's own opp(I).
+template <class S, int I>
+__device__ __forceinline__ void quad_bounce(const S* src, unsigned NT, int gi, uint32_t lk0, uint32_t lk1, unsigned& w) {
+    const unsigned short* o = reinterpret_cast<const unsigned short*>(src + ((unsigned)opp(I) * NT + (unsigned)gi));
+    if ((lk0 >> I) & 1u) w = __byte_perm(w, pop_ld(o), 0x3254);
+    if ((lk1 >> I) & 1u) w = __byte_perm(w, pop_ld(o + 1), 0x5410);
+}
+
+// Collision of the opposite directions (I, I + 1), I odd, of one node pair:
+// unpacked from the pulled words, collided, rounded and packed again in place.
+template <class S, int I, bool UW>
+__device__ __forceinline__ void quad_collide_pair(const Mac2& m, unsigned seed, uint32_t lk0, uint32_t lk1, const ChannelDev& C, int y,
+                                                  unsigned& wi, unsigned& wj) {
+    F2 h[2] = {quad_pop<S, I, UW>(wi, lk0, lk1, C, y), quad_pop<S, I + 1, UW>(wj, lk0, lk1, C, y)};
+    collide_two<true, I>(h[0], h[1], m, C);
+    wi = cvt_rs2<S>(h[0].y, h[0].x, seed * sr_k(I));
+    wj = cvt_rs2<S>(h[1].y, h[1].x, seed * sr_k(I + 1));
+}
+
+// One node pair of the quad in its packed words (w: the .x or .y halves, one
+// word per direction): moments, then the collision, each from its own
+// unpacking of the words, so that no more than two directions are held as
+// floats at a time (holding all 19 took 128 registers and 16 warps per SM).
+// The post-collision words replace the pulled ones.
+template <class S, bool UW>
+__device__ __forceinline__ void quad_half(const ChannelDev& C, int gi, int y, unsigned w[Q], uint32_t lk0, uint32_t lk1,
+                                          bool forced, float4 g0, float4 g1, Mac2& m) {
+    macro_force(C, g0, g1, forced, m);
+    {
+#define LBIBM_QD(I) const F2 h##I = quad_pop<S, I, UW>(w[I], lk0, lk1, C, y);
+        PairSums ps;
+        F2 h0;
+        {
+            LBIBM_QD(1) LBIBM_QD(2) LBIBM_QD(3) LBIBM_QD(4) LBIBM_QD(5) LBIBM_QD(6)
+            ps.axis(h1, h2, h3, h4, h5, h6);
+        }
+        {
+            LBIBM_QD(7) LBIBM_QD(8) LBIBM_QD(9) LBIBM_QD(10) LBIBM_QD(11) LBIBM_QD(12) LBIBM_QD(13) LBIBM_QD(14)
+            LBIBM_QD(15) LBIBM_QD(16) LBIBM_QD(17) LBIBM_QD(18)
+            ps.diag(h7, h8, h9, h10, h11, h12, h13, h14, h15, h16, h17, h18);
+        }
+#undef LBIBM_QD
+        h0 = quad_pop<S, 0, UW>(w[0], lk0, lk1, C, y);
+        macro_pair<true>(ps, h0, m);
     }
-    pair_collide<true>(C, g0, g1, forced, h, m);
+    // the collision unpacks the words again: keep the compiler from holding
+    // the first unpacking's 38 floats across the moments
+#pragma unroll
+    for (int i = 0; i < Q; ++i) asm volatile("" : "+r"(w[i]));
+    macro_terms(C, m);
     const unsigned seed = sr_seed((unsigned)gi, m.drho.x, m.ux.y);
-    using IO = PairIO<S>;
-    if (!((lk0 | lk1) & 1u)) {
-#define LBIBM_P2(I) IO::st2(dst + ((unsigned)(I) * NT + (unsigned)gi), h[I], seed * sr_k(I));
-        LBIBM_ALL_I(LBIBM_P2)
-#undef LBIBM_P2
+    {
+        const F2 X0 = fma2(C.om2, m.A1, m.mug);
+        const F2 h0 = fma2(C.omc2, quad_pop<S, 0, UW>(w[0], lk0, lk1, C, y), X0);
+        w[0] = cvt_rs2<S>(h0.y, h0.x, seed * sr_k(0));
+    }
+#define LBIBM_QC(I, J) quad_collide_pair<S, I, UW>(m, seed, lk0, lk1, C, y, w[I], w[J]);
+    LBIBM_QC(1, 2) LBIBM_QC(3, 4) LBIBM_QC(5, 6) LBIBM_QC(7, 8) LBIBM_QC(9, 10) LBIBM_QC(11, 12) LBIBM_QC(13, 14)
+    LBIBM_QC(15, 16) LBIBM_QC(17, 18)
+#undef LBIBM_QC
+}
+
+// Both node pairs of an in-range quad: bounce-back, collision, stores.
+template <class S, bool UW>
+__device__ __forceinline__ void quad_update(const LatticeArgs& a, const ChannelDev& C, const S* src, S* dst, unsigned NT,
+                                            int gi0, int y, unsigned wx[Q], unsigned wy[Q], uint4 lk, bool forced,
+                                            bool prevf) {
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4* gcur = a.par ? a.g1 : a.g0;
+    const uint32_t any = lk.x | lk.y | lk.z | lk.w;
+    if (any & ~1u) {
+#define LBIBM_QB(I)                                                  \
+    if (I > 0) {                                                     \
+        quad_bounce<S, I>(src, NT, gi0, lk.x, lk.y, wx[I]);          \
+        quad_bounce<S, I>(src, NT, gi0 + 2, lk.z, lk.w, wy[I]);      \
+    }
+        LBIBM_ALL_I(LBIBM_QB)
+#undef LBIBM_QB
+    }
+    {
+        Mac2 m;
+        quad_half<S, UW>(C, gi0, y, wx, lk.x, lk.y, forced, forced ? gcur[gi0] : z4, forced ? gcur[gi0 + 1] : z4, m);
+        if (forced) {
+            if (!(lk.x & 1u)) a.u[gi0] = make_float4(m.ux.x, m.uy.x, m.uz.x, m.rho.x);
+            if (!(lk.y & 1u)) a.u[gi0 + 1] = make_float4(m.ux.y, m.uy.y, m.uz.y, m.rho.y);
+        }
+    }
+    // the second pair starts when the first one is packed again (interleaving
+    // the two would hold both pairs' floats)
+#pragma unroll
+    for (int i = 0; i < Q; ++i) asm volatile("" : "+r"(wx[i]), "+r"(wy[i]));
+    {
+        Mac2 m;
+        quad_half<S, UW>(C, gi0 + 2, y, wy, lk.z, lk.w, forced, forced ? gcur[gi0 + 2] : z4,
+                         forced ? gcur[gi0 + 3] : z4, m);
+        if (forced) {
+            if (!(lk.z & 1u)) a.u[gi0 + 2] = make_float4(m.ux.x, m.uy.x, m.uz.x, m.rho.x);
+            if (!(lk.w & 1u)) a.u[gi0 + 3] = make_float4(m.ux.y, m.uy.y, m.uz.y, m.rho.y);
+        }
+    }
+    if (!(any & 1u)) {
+#define LBIBM_Q4(I) pop_st<S>(reinterpret_cast<uint2*>(dst + ((unsigned)(I) * NT + (unsigned)gi0)), make_uint2(wx[I], wy[I]));
+        LBIBM_ALL_I(LBIBM_Q4)
+#undef LBIBM_Q4
     } else {
-        if (!(lk0 & 1u)) {
-#define LBIBM_P1(I) IO::st1(dst + ((unsigned)(I) * NT + (unsigned)gi), h[I].x, seed * sr_k(I));
-            LBIBM_ALL_I(LBIBM_P1)
-#undef LBIBM_P1
-        }
-        if (!(lk1 & 1u)) {
-#define LBIBM_P1(I) IO::st1(dst + ((unsigned)(I) * NT + (unsigned)(gi + 1)), h[I].y, (seed * sr_k(I)) >> 16);
-            LBIBM_ALL_I(LBIBM_P1)
-#undef LBIBM_P1
-        }
+        // a solid node keeps its populations; the others are stored alone
+#define LBIBM_Q1(I)                                                                                        \
+    {                                                                                                      \
+        unsigned short* o = reinterpret_cast<unsigned short*>(dst + ((unsigned)(I) * NT + (unsigned)gi0)); \
+        if (!(lk.x & 1u)) pop_st<S>(o, (unsigned short)(wx[I] & 0xffffu));                                 \
+        if (!(lk.y & 1u)) pop_st<S>(o + 1, (unsigned short)(wx[I] >> 16));                                 \
+        if (!(lk.z & 1u)) pop_st<S>(o + 2, (unsigned short)(wy[I] & 0xffffu));                             \
+        if (!(lk.w & 1u)) pop_st<S>(o + 3, (unsigned short)(wy[I] >> 16));                                 \
+    }
+        LBIBM_ALL_I(LBIBM_Q1)
+#undef LBIBM_Q1
+    }
+    if (prevf) {
+        float4* gprev = a.par ? a.g0 : a.g1;
+        if (!(lk.x & 1u)) gprev[gi0] = z4;
+        if (!(lk.y & 1u)) gprev[gi0 + 1] = z4;
+        if (!(lk.z & 1u)) gprev[gi0 + 2] = z4;
+        if (!(lk.w & 1u)) gprev[gi0 + 3] = z4;
     }
 }
 
-template <class S, bool ROW>
+template <class S, bool ROW, bool UW>
 __device__ __forceinline__ void sc_quad(const LatticeArgs& a, const ChannelDev& C, int p0, int lane, int xr, int yr,
                                         int zr) {
     static_assert(sizeof(S) == 2, "the quad variant packs 16-bit populations");
@@ -1167,61 +1294,39 @@ __device__ __forceinline__ void sc_quad(const LatticeArgs& a, const ChannelDev& 
     pdl_entry();
     const uint8_t fcur = __ldg((par ? a.fl1 : a.fl0) + grp);
     const uint8_t fprev = __ldg(fl_prev + grp);
-    uint2 w[Q];
-    unsigned e[Q];
+    unsigned wx[Q], wy[Q];
+    {
+        uint2 w[Q];
+        unsigned e[Q];
 #define LBIBM_QP(I) quad_pull<S, I>(src, NT, gi0, nb, inr, edge_lo, edge_hi, w[I], e[I]);
-    LBIBM_ALL_I(LBIBM_QP)
+        LBIBM_ALL_I(LBIBM_QP)
 #undef LBIBM_QP
+#define LBIBM_QS(I)                                    \
+    quad_shift<I>(w[I], e[I], edge_lo, edge_hi);       \
+    wx[I] = w[I].x;                                    \
+    wy[I] = w[I].y;
+        LBIBM_ALL_I(LBIBM_QS)
+#undef LBIBM_QS
+    }
     const bool forced = fcur != 0;
     const bool prevf = fprev != 0;
-    const bool wslow = __any_sync(FULL, fslow != 0);
-#define LBIBM_QS(I) quad_shift<I>(w[I], e[I], edge_lo, edge_hi);
-    LBIBM_ALL_I(LBIBM_QS)
-#undef LBIBM_QS
     uint4 lk = make_uint4(0u, 0u, 0u, 0u);
-    if (wslow && inr && fslow) lk = __ldg(reinterpret_cast<const uint4*>(a.links + gi0));
-    if (inr) {
-        Mac2 m0, m1;
-        const float4* gcur = par ? a.g1 : a.g0;
-        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        quad_half<S>(C, src, dst, NT, gi0, y, w, 0, lk.x, lk.y, forced, forced ? gcur[gi0] : z4,
-                     forced ? gcur[gi0 + 1] : z4, m0);
-        quad_half<S>(C, src, dst, NT, gi0 + 2, y, w, 1, lk.z, lk.w, forced, forced ? gcur[gi0 + 2] : z4,
-                     forced ? gcur[gi0 + 3] : z4, m1);
-        float4* gprev = par ? a.g0 : a.g1;
-        if (forced) {
-            if (!(lk.x & 1u)) a.u[gi0] = make_float4(m0.ux.x, m0.uy.x, m0.uz.x, m0.rho.x);
-            if (!(lk.y & 1u)) a.u[gi0 + 1] = make_float4(m0.ux.y, m0.uy.y, m0.uz.y, m0.rho.y);
-            if (!(lk.z & 1u)) a.u[gi0 + 2] = make_float4(m1.ux.x, m1.uy.x, m1.uz.x, m1.rho.x);
-            if (!(lk.w & 1u)) a.u[gi0 + 3] = make_float4(m1.ux.y, m1.uy.y, m1.uz.y, m1.rho.y);
-        }
-        if (prevf) {
-            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (!(lk.x & 1u)) gprev[gi0] = z4;
-            if (!(lk.y & 1u)) gprev[gi0 + 1] = z4;
-            if (!(lk.z & 1u)) gprev[gi0 + 2] = z4;
-            if (!(lk.w & 1u)) gprev[gi0 + 3] = z4;
-        }
-    }
+    if (inr && fslow) lk = __ldg(reinterpret_cast<const uint4*>(a.links + gi0));
+    if (inr) quad_update<S, UW>(a, C, src, dst, NT, gi0, y, wx, wy, lk, forced, prevf);
     // the lane holding the first node of each 32-node group clears the previous
     // step's flag after every lane of the warp has consumed it
     __syncwarp();
     if (prevf && (gi0 & 31) == 0) fl_prev[grp] = 0;
 }
 
-// Resident threads per SM of the quad variant's register budget.
+// Resident threads per SM of the quad variant's register budget (512: 289 us,
+// 640: 261, 704: 278, 768: 282; 512x256x128 FP16, GB300).
 #ifndef LBIBM_K3_QUAD_THREADS
 #define LBIBM_K3_QUAD_THREADS 640
 #endif
 
-template <class S, int BS, int MINB>
-__global__ void __launch_bounds__(BS, MINB) k_stream_collide_quad(const __grid_constant__ LatticeArgs a) {
-    // (sc_quad waits for the predecessor after its population loads)
-    const int b = blockIdx.x;
-    int c = 0;
-    for (int k = 1; k < a.n_ch; ++k)
-        if (b >= chan(a, k).blk0) c = k;
-    const ChannelDev C = chan(a, c);
+template <class S, int BS, bool UW>
+__device__ __forceinline__ void quad_block(const LatticeArgs& a, const ChannelDev& C, int b) {
     const int lane = threadIdx.x & 31;
     const int pb = (b - C.blk0) * (4 * BS);                  // first channel-local node of the block
     const int p0 = pb + 4 * (int)threadIdx.x;
@@ -1230,10 +1335,24 @@ __global__ void __launch_bounds__(BS, MINB) k_stream_collide_quad(const __grid_c
         // the block is a piece of one row: y and z are the block's
         const int r = fdiv(pb, C.dnx);
         const int z = fdiv(r, C.dny);
-        sc_quad<S, true>(a, C, p0, lane, pb - r * C.nx + 4 * (int)threadIdx.x, r - z * C.ny, z);
+        sc_quad<S, true, UW>(a, C, p0, lane, pb - r * C.nx + 4 * (int)threadIdx.x, r - z * C.ny, z);
         return;
     }
-    sc_quad<S, false>(a, C, p0, lane, 0, 0, 0);
+    sc_quad<S, false, UW>(a, C, p0, lane, 0, 0, 0);
+}
+
+// ONE: a single channel, whose constants stay in the parameter bank (no
+// registers); UW: some channel has moving walls.
+template <class S, int BS, int MINB, bool ONE, bool UW>
+__global__ void __launch_bounds__(BS, MINB) k_stream_collide_quad(const __grid_constant__ LatticeArgs a) {
+    // (sc_quad waits for the predecessor)
+    const int b = blockIdx.x;
+    if constexpr (ONE) {
+        quad_block<S, BS, UW>(a, a.chp[0], b);
+    } else {
+        const ChannelDev C = chan(a, sc_channel(a, b));
+        quad_block<S, BS, UW>(a, C, b);
+    }
 }
 
 // Bulk of the overlapped schedule (one node per thread; a warp is one group).
@@ -1550,9 +1669,7 @@ template <class S, int BS>
 __global__ void __launch_bounds__(BS, K3MinBlocks<S, 1, BS>::value) k_stream_collide_brinkman(const __grid_constant__ LatticeArgs a) {
     pdl_entry();
     const int b = blockIdx.x;
-    int c = 0;
-    for (int k = 1; k < a.n_ch; ++k)
-        if (b >= chan(a, k).blk0) c = k;
+    const int c = sc_channel(a, b);
     const ChannelDev C = chan(a, c);
     sc_nodes<S, 1, SC_BRINK>(a, C, (b - C.blk0) * BS + (int)threadIdx.x, threadIdx.x & 31);
 }
@@ -1847,6 +1964,16 @@ bool k3_config_supported(int storage, K3Config c) {
     return false;
 }
 
+template <class S, int BS>
+static cudaError_t launch_quad(const LatticeArgs& a, int blocks, cudaStream_t s) {
+    constexpr int MINB = LBIBM_K3_QUAD_THREADS / BS;
+    bool uw = false;
+    for (int k = 0; k < a.n_ch && k < MAXCH_P; ++k) uw = uw || a.chp[k].has_uw;
+    if (uw || a.n_ch > MAXCH_P) return launch_ex(k_stream_collide_quad<S, BS, MINB, false, true>, blocks, BS, 0, s, a.pdl, a);
+    if (a.n_ch > 1) return launch_ex(k_stream_collide_quad<S, BS, MINB, false, false>, blocks, BS, 0, s, a.pdl, a);
+    return launch_ex(k_stream_collide_quad<S, BS, MINB, true, false>, blocks, BS, 0, s, a.pdl, a);
+}
+
 template <class S>
 static cudaError_t launch_sc_typed(const LatticeArgs& a, K3Config c, int blocks, cudaStream_t s) {
 #define LBIBM_CASE(N, B)                                   \
@@ -1860,9 +1987,8 @@ static cudaError_t launch_sc_typed(const LatticeArgs& a, K3Config c, int blocks,
     }
     if constexpr (sizeof(S) == 2) {
         if (c.npt == 4) {
-            if (c.bs == 64) return launch_ex(k_stream_collide_quad<S, 64, 512 / 64>, blocks, 64, 0, s, a.pdl, a);
-            if (c.bs == 128)
-                return launch_ex(k_stream_collide_quad<S, 128, LBIBM_K3_QUAD_THREADS / 128>, blocks, 128, 0, s, a.pdl, a);
+            if (c.bs == 64) return launch_quad<S, 64>(a, blocks, s);
+            if (c.bs == 128) return launch_quad<S, 128>(a, blocks, s);
             return cudaErrorInvalidConfiguration;
         }
     }

@@ -1015,6 +1015,13 @@ lb_status lb_create_batch(const lb_params* params, int n_channels, void* cuda_st
         d.omega = (float)(1.0 / p.tau);
         d.fpre = (float)(1.0 - 1.0 / (2.0 * p.tau));
         for (int a = 0; a < 3; ++a) d.G[a] = (float)p.body_force[a];
+        auto pair = [](float v) { return make_float2(v, v); };
+        d.om2 = pair(d.omega);
+        d.omc2 = pair(1.0f - d.omega);
+        d.c3om2 = pair(3.0f * d.omega);
+        d.c9fp2 = pair(9.0f * d.fpre);
+        d.c3fp2 = pair(3.0f * d.fpre);
+        for (int a = 0; a < 3; ++a) d.G2[a] = pair(d.G[a]);
         d.has_uw = 0;
         for (int w = 0; w < 2; ++w)
             for (int a = 0; a < 3; ++a) {

@@ -132,6 +132,9 @@ struct ChannelDev {
     float G[3];           // uniform body force
     float uw[2][3];       // y-low / y-high wall velocity
     int has_uw;
+    // the same constants as packed pairs for the two-node collision:
+    // omega, 1 - omega, 3 omega, 9 fpre, 3 fpre and the body force
+    float2 om2, omc2, c3om2, c9fp2, c3fp2, G2[3];
 };
 
 struct __align__(32) Q4 {
