@@ -247,9 +247,11 @@ lb_status lb_get_kernel_config(lb_ctx* ctx, int* nodes_per_thread, int* block_si
  * populations (every direction's plane) of the nodes nodes_ahead past its
  * own, so that blocks running later find their pulls in L2 rather than in
  * HBM.  A performance setting only (Sec. 2.1's update is unchanged; results
- * are bit-identical for every distance).  0 = off (the default); otherwise a
- * multiple of 256 up to 2^24, else LB_ERR_ARG.  The bound on the useful
- * distance is the L2 (19 x 4 bytes per node of distance for FP32 storage). */
+ * are bit-identical for every distance).  0 (the default): the library's own
+ * distance, five megabytes of populations (65,536 nodes in FP32, 131,072 in
+ * 16 bits); otherwise a multiple of 256 up to 2^24, else LB_ERR_ARG.  The
+ * bound on the useful distance is the L2 (19 x 4 bytes per node of distance
+ * for FP32 storage). */
 lb_status lb_set_prefetch(lb_ctx* ctx, int nodes_ahead);
 lb_status lb_get_prefetch(lb_ctx* ctx, int* nodes_ahead);
 

@@ -175,8 +175,8 @@ __device__ __forceinline__ const ChannelDev& chan(const LatticeArgs& a, int c) {
 template <class S>
 __device__ __forceinline__ void prefetch_ahead(const LatticeArgs& a, long long g0, int nb) {
     if (a.pf_nodes <= 0 || threadIdx.x >= Q) return;
-    const long long g = g0 + a.pf_nodes;
-    if (g >= a.Ntot) return;
+    const long long g = a.rev ? g0 - a.pf_nodes : g0 + a.pf_nodes;
+    if (g < 0 || g >= a.Ntot) return;
     const long long n = a.Ntot - g < nb ? a.Ntot - g : nb;
     const S* src = (const S*)(a.par ? a.h1 : a.h0) + (size_t)threadIdx.x * (size_t)a.Ntot + g;
     const unsigned bytes = (unsigned)(n * (long long)sizeof(S)) & ~15u;
@@ -466,22 +466,18 @@ __device__ __forceinline__ void bounce_back(const S* src, long long NT, int gi, 
 }
 
 // Resident threads per SM the register budget is sized for.  One node per
-// thread: 1152 threads (56 registers) for FP32 and for 16-bit populations, the
-// fastest of the budgets measured on GB300 with row-aligned blocks (FP32: 1280
-// 61.0 us, 1152 60.6, 1024 64.1; 16-bit: 1280 56.2, 1152 55.9, 1024 58.3); two
-// nodes per thread: 512 (128 registers); four: 256 (255 registers).
-#ifndef LBIBM_K3_THREADS1
-#define LBIBM_K3_THREADS1 1152
-#endif
-#ifndef LBIBM_K3_THREADS1_16
-#define LBIBM_K3_THREADS1_16 1152
-#endif
-#ifndef LBIBM_K3_THREADS2
-#define LBIBM_K3_THREADS2 512
-#endif
+// thread: 1152 threads (56 registers); two nodes per thread: 512 (128
+// registers); four: 256 (255 registers).  (256x128x64 on GB300: FP32 1280 61.0
+// us, 1152 60.6, 1024 64.1; 16-bit: 1280 56.2, 1152 55.9, 1024 58.3.)  The
+// WIDE form of the FP32 kernel, one channel with its constants in the parameter
+// bank, fits 1280 threads (48 registers) without spilling: 256x128x64 57.2
+// against 58.0 us, 512x256x128 409 against 411-418, while lattices of a few
+// waves wait on each warp's latency, which the smaller budget lengthens
+// (96x48x32 reproducible cycle 18.8 -> 19.1 us, 128x64x64 differentiable 1 %),
+// so it takes over from WIDE_BLOCKS blocks of 128 on (six waves).
+constexpr int WIDE_BLOCKS = 8192;
 template <class S, int NPT, int BS> struct K3MinBlocks {
-    static constexpr int threads = NPT == 1 ? (sizeof(S) == 4 ? LBIBM_K3_THREADS1 : LBIBM_K3_THREADS1_16)
-                                            : (NPT == 2 ? LBIBM_K3_THREADS2 : 256);
+    static constexpr int threads = NPT == 1 ? 1152 : (NPT == 2 ? 512 : 256);
     static constexpr int value = threads / BS > 0 ? threads / BS : 1;
 };
 
@@ -611,6 +607,13 @@ __device__ __forceinline__ void sc_nodes(const LatticeArgs& a, const ChannelDev&
     if (prevf && (gp0 & 31) == 0) fl_prev[grp] = 0;
 }
 
+// Traversal of one stream-collide launch: backwards when the host asks for it
+// (odd steps of lattices near the size of L2, whose last-written populations
+// are then read first).
+__device__ __forceinline__ int sc_block(const LatticeArgs& a) {
+    return a.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+}
+
 // Channel of block b: the last one whose first block is <= b (bisection; the
 // linear search cost the 24-channel sweep 40 of 388 us, GB300).
 __device__ __forceinline__ int sc_channel(const LatticeArgs& a, int b) {
@@ -624,11 +627,7 @@ __device__ __forceinline__ int sc_channel(const LatticeArgs& a, int b) {
 }
 
 template <class S, int NPT, int BS>
-__global__ void __launch_bounds__(BS, K3MinBlocks<S, NPT, BS>::value) k_stream_collide(const __grid_constant__ LatticeArgs a) {
-    // (sc_nodes waits for the predecessor after its population loads)
-    const int b = blockIdx.x;
-    const int c = sc_channel(a, b);
-    const ChannelDev C = chan(a, c);   // registers: read once from the parameter bank
+__device__ __forceinline__ void sc_block_nodes(const LatticeArgs& a, const ChannelDev& C, int b) {
     const int lane = threadIdx.x & 31;
     const int p0 = ((b - C.blk0) * BS + (int)threadIdx.x) * NPT;   // first channel-local node of this thread
     prefetch_ahead<S>(a, C.base + (long long)(b - C.blk0) * BS * NPT, BS * NPT);
@@ -645,6 +644,20 @@ __global__ void __launch_bounds__(BS, K3MinBlocks<S, NPT, BS>::value) k_stream_c
         }
     }
     sc_nodes<S, NPT, SC_ALL>(a, C, p0, lane);
+}
+
+// ONE: a single channel, whose constants stay in the parameter bank (which is
+// what lets FP32 run in 48 registers).
+template <class S, int NPT, int BS, bool ONE, bool WIDE>
+__global__ void __launch_bounds__(BS, WIDE ? 1280 / BS : K3MinBlocks<S, NPT, BS>::value) k_stream_collide(const __grid_constant__ LatticeArgs a) {
+    // (sc_nodes waits for the predecessor after its population loads)
+    const int b = sc_block(a);
+    if constexpr (ONE) {
+        sc_block_nodes<S, NPT, BS>(a, a.chp[0], b);
+    } else {
+        const ChannelDev C = chan(a, sc_channel(a, b));   // registers: read once from the parameter bank
+        sc_block_nodes<S, NPT, BS>(a, C, b);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1018,7 +1031,7 @@ __device__ __forceinline__ void sc_pair(const LatticeArgs& a, const ChannelDev& 
 template <class S, int BS>
 __global__ void __launch_bounds__(BS, LBIBM_K3_PAIR_THREADS / BS) k_stream_collide_pair(const __grid_constant__ LatticeArgs a) {
     // (sc_pair waits for the predecessor after its population loads)
-    const int b = blockIdx.x;
+    const int b = sc_block(a);
     const int c = sc_channel(a, b);
     const ChannelDev C = chan(a, c);
     const int pb = (b - C.blk0) * (2 * BS);                  // first channel-local node of the block
@@ -1346,7 +1359,7 @@ __device__ __forceinline__ void quad_block(const LatticeArgs& a, const ChannelDe
 template <class S, int BS, int MINB, bool ONE, bool UW>
 __global__ void __launch_bounds__(BS, MINB) k_stream_collide_quad(const __grid_constant__ LatticeArgs a) {
     // (sc_quad waits for the predecessor)
-    const int b = blockIdx.x;
+    const int b = sc_block(a);
     if constexpr (ONE) {
         quad_block<S, BS, UW>(a, a.chp[0], b);
     } else {
@@ -1668,7 +1681,7 @@ __global__ void __launch_bounds__(BS, 512 / BS) k_stream_collide_pipe(const __gr
 template <class S, int BS>
 __global__ void __launch_bounds__(BS, K3MinBlocks<S, 1, BS>::value) k_stream_collide_brinkman(const __grid_constant__ LatticeArgs a) {
     pdl_entry();
-    const int b = blockIdx.x;
+    const int b = sc_block(a);
     const int c = sc_channel(a, b);
     const ChannelDev C = chan(a, c);
     sc_nodes<S, 1, SC_BRINK>(a, C, (b - C.blk0) * BS + (int)threadIdx.x, threadIdx.x & 31);
@@ -1964,6 +1977,15 @@ bool k3_config_supported(int storage, K3Config c) {
     return false;
 }
 
+// One node per thread, one channel.
+template <class S, int BS>
+static cudaError_t launch_one(const LatticeArgs& a, int blocks, cudaStream_t s) {
+    if constexpr (sizeof(S) == 4 && BS == 128) {
+        if (blocks >= WIDE_BLOCKS) return launch_ex(k_stream_collide<S, 1, BS, true, true>, blocks, BS, 0, s, a.pdl, a);
+    }
+    return launch_ex(k_stream_collide<S, 1, BS, true, false>, blocks, BS, 0, s, a.pdl, a);
+}
+
 template <class S, int BS>
 static cudaError_t launch_quad(const LatticeArgs& a, int blocks, cudaStream_t s) {
     constexpr int MINB = LBIBM_K3_QUAD_THREADS / BS;
@@ -1978,7 +2000,8 @@ template <class S>
 static cudaError_t launch_sc_typed(const LatticeArgs& a, K3Config c, int blocks, cudaStream_t s) {
 #define LBIBM_CASE(N, B)                                   \
     if (c.npt == N && c.bs == B) {                         \
-        return launch_ex(k_stream_collide<S, N, B>, blocks, B, 0, s, a.pdl, a); \
+        if (N == 1 && a.n_ch == 1) return launch_one<S, B>(a, blocks, s); \
+        return launch_ex(k_stream_collide<S, N, B, false, false>, blocks, B, 0, s, a.pdl, a); \
     }
     if (c.npt == 2) {
         if (c.bs == 128) return launch_ex(k_stream_collide_pair<S, 128>, blocks, 128, 0, s, a.pdl, a);

@@ -191,7 +191,7 @@ struct lb_ctx {
         double *lam_c = nullptr, *grad = nullptr;
     } adj;
     int bulk_res = 10;             // resident bulk blocks per SM (128 threads)
-    int pf_nodes = 0;              // stream-collide L2 prefetch distance (lattice nodes, 0 = off)
+    int pf_nodes = 0;              // stream-collide L2 prefetch distance (lattice nodes, 0: PREFETCH_BYTES)
     long long smem_per_sm = 0;
     // timing
     int timing = 0;          // bit k: record events around kernel class k (no graph)
@@ -300,6 +300,20 @@ __global__ void k_guard_count(const unsigned char* __restrict__ p, size_t n, uns
 
 size_t pop_bytes(lb_storage s) { return s == LB_F32 ? 4 : 2; }
 
+// The stream-collide's own L2 prefetch distance (lb_set_prefetch 0): five
+// megabytes of populations, 65,536 nodes in FP32 and 131,072 in 16 bits, about
+// what the resident blocks hold in flight (GB300, without / with: 256x128x64
+// FP32 60.0 / 57.2 us, 512x256x128 FP32 411 / 409, FP16 261 / 246; half the
+// distance 1-4 us slower, twice no faster).
+constexpr int PREFETCH_BYTES = Q * 65536 * 4;
+// Odd steps walk the blocks backwards when both population buffers together
+// are about the size of L2 (126 MB, three quarters to three halves): they then
+// begin with what the previous step wrote last.  Measured on GB300: 181x75x53
+// FP32, 110 MB, 36.3 -> 35.3 us per cycle; 256x128x64 FP32, 319 MB, 70.4 ->
+// 71.2; populations that stay in L2 anyway lose the die they lie on (32x16x64,
+// 5 MB: 11.7 -> 12.7; 128x64x64 differentiable, 80 MB, 1 % slower).
+constexpr size_t ZIGZAG_MIN = (size_t)94 << 20, ZIGZAG_MAX = (size_t)189 << 20;
+
 LatticeArgs lattice_args(const lb_ctx* ctx, int par) {
     LatticeArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -327,7 +341,10 @@ LatticeArgs lattice_args(const lb_ctx* ctx, int par) {
     a.dlist = ctx->dlist[par];
     a.dcount = ctx->dcount ? ctx->dcount + par : nullptr;
     a.tma_err = ctx->sched_err ? ctx->sched_err + 1 : nullptr;
-    a.pf_nodes = ctx->pf_nodes;
+    a.pf_nodes = ctx->pf_nodes > 0 ? ctx->pf_nodes : PREFETCH_BYTES / (Q * (int)pop_bytes(ctx->storage));
+    if (a.pf_nodes >= ctx->Ntot) a.pf_nodes = 0;   // nothing that far ahead
+    const size_t pops = 2 * (size_t)Q * ctx->plane * pop_bytes(ctx->storage);
+    a.rev = par && !ctx->phi && pops >= ZIGZAG_MIN && pops <= ZIGZAG_MAX;
     return a;
 }
 

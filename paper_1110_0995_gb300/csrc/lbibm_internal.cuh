@@ -185,6 +185,7 @@ struct LatticeArgs {
     // asks L2 for the source rows of the nodes pf_nodes past its own, so the
     // blocks that run a wave later find them there instead of in DRAM.
     int pf_nodes;
+    int rev;              // stream-collide: walk the blocks backwards
     ChannelDev chp[MAXCH_P];   // copy of the first channels (constant bank)
 };
 
