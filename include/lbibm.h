@@ -398,7 +398,8 @@ lb_status bead_forces(const double* xyz, const double* moments, int n, const bea
  * axes; xyz (n x 3, host) is updated in place.  Errors as bead_forces. */
 lb_status bead_relax(double* xyz, const double* moments, int n, const bead_params* p, int steps, void* cuda_stream);
 
-/* Conservation diagnostics of the selected channel, FP64 on the device:
+/* Conservation diagnostics of the selected channel (sums exact in 2^-56 fixed
+ * point or FP64, on the device):
  * out[0] = sum of rho over fluid nodes, out[1..3] = sum of sum_i e_i f_i
  * after the last collision, out[4] = number of non-finite populations,
  * out[5] = max |u| over fluid nodes.  Returns LB_ERR_NUMERIC when out[4] > 0

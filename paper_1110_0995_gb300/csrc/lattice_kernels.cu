@@ -20,6 +20,7 @@
 
 #include <cuda_pipeline.h>
 
+#include <algorithm>
 #include <type_traits>
 
 namespace lbibm {
@@ -2330,11 +2331,22 @@ cudaError_t launch_pull_populations(const LatticeArgs& a, int c, float* h_out, c
 }
 
 // ---------------------------------------------------------------------------
-// Conservation diagnostics: FP64 per-thread sums, FP64 block reduction, one
-// partial per block, then an ordered final sum (deterministic).
+// Conservation diagnostics, one pass over the populations.  What bounds it
+// besides reading them is this GPU's FP64 pipe (two operations per clock per
+// SM), so the nodes' part runs without it:
+//   * rho - 1 and the momentum are added as 64-bit integers in 2^-56 units
+//     (each FP32 moment rounded once, far below its own rounding; the sums are
+//     exact), for moments below 1, at most 64 nodes before they move to FP64;
+//   * the fastest node is found by comparing |v|^2 / rho^2 as pairs of FP32
+//     numbers (about 2^-44 relative), and only its speed is evaluated in FP64;
+//   * a node outside those ranges (a run that is blowing up) takes the FP64
+//     path by itself.
+// The last block to finish adds the blocks' FP64 partials in a fixed order.
+// Measured on GB300 (whole call, with FP64 arithmetic per node, a serial final
+// sum in a second launch and three copies before): 512x256x128 FP32 1858 -> 302
+// us (reading alone 188), 256x128x64 340 -> 68, 96x40x32 180 -> 35.
 // ---------------------------------------------------------------------------
 constexpr int DIAG_BLOCK = 256;
-constexpr int DIAG_N = 6;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -2347,71 +2359,241 @@ __device__ __forceinline__ double warp_max(double v) {
     return v;
 }
 
+// round(v 2^56) for |v| < 1: v 2^28 = m + f, both exact in FP32.
+__device__ __forceinline__ long long diag_fixed(float v) {
+    const float s = v * 268435456.0f;
+    const float m = rintf(s);
+    const float f = (s - m) * 268435456.0f;
+    return ((long long)__float2int_rn(m) << 28) + (long long)__float2int_rn(f);
+}
+
+// An unevaluated sum hi + lo of two FP32 numbers.
+struct Two {
+    float hi, lo;
+};
+__device__ __forceinline__ Two two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return Two{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Two two_sqr(Two a) {
+    const float p = __fmul_rn(a.hi, a.hi);
+    return Two{p, fmaf(2.0f * a.hi, a.lo, fmaf(a.hi, a.hi, -p))};
+}
+__device__ __forceinline__ Two two_add(Two a, Two b) {
+    const Two s = two_sum(a.hi, b.hi);
+    return two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+// a / b, b > 0
+__device__ __forceinline__ Two two_div(Two a, Two b) {
+    const float q = __fdiv_rn(a.hi, b.hi);
+    const float r = fmaf(-q, b.lo, fmaf(-q, b.hi, a.hi) + a.lo);
+    return two_sum(q, __fdiv_rn(r, b.hi));
+}
+__device__ __forceinline__ bool two_less(Two a, Two b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
+
+// Speed of one node in FP64 from its moments and force (infinite when it is not a number).
+__device__ __forceinline__ double diag_speed(float drho, float jx, float jy, float jz, float gx, float gy, float gz) {
+    const double rho = 1.0 + (double)drho;
+    const double ux = (jx - 0.5 * gx) / rho, uy = (jy - 0.5 * gy) / rho, uz = (jz - 0.5 * gz) / rho;
+    const double um = sqrt(ux * ux + uy * uy + uz * uz);
+    return (um != um) ? INFINITY : um;
+}
+
 template <class S>
-__global__ void __launch_bounds__(DIAG_BLOCK) k_diag_partial(const __grid_constant__ LatticeArgs a, int c,
-                                                             double* partials) {
+__device__ __forceinline__ void diag_moments(const LatticeArgs& a, const S* hs, long long gp, float h[Q], float& drho,
+                                             float& jx, float& jy, float& jz) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) h[i] = Pop<S>::ld(hs, (long long)i * a.Ntot + gp, i);
+    moments(h, drho, jx, jy, jz);
+}
+
+__device__ __forceinline__ void diag_force(const LatticeArgs& a, const ChannelDev& C, long long gp, float& gx, float& gy,
+                                           float& gz) {
+    gx = C.G[0]; gy = C.G[1]; gz = C.G[2];
+    if ((a.par ? a.fl0 : a.fl1)[gp >> 5]) {
+        const float4 g = (a.par ? a.g0 : a.g1)[gp];
+        gx += g.x; gy += g.y; gz += g.z;
+    }
+}
+
+// One block's share of the result: FP64 sums of rho and momentum, the
+// non-finite populations, the largest speed of the nodes that took the FP64
+// path, and the fastest other node.
+struct DiagPartial {
+    double s[4];
+    double bad, fast;
+    Two best;
+    long long node;   // -1: none
+};
+
+__device__ __forceinline__ void diag_merge(DiagPartial& p, const DiagPartial& q) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p.s[k] += q.s[k];
+    p.bad += q.bad;
+    p.fast = fmax(p.fast, q.fast);
+    if (q.node >= 0 && (p.node < 0 || two_less(p.best, q.best))) {
+        p.best = q.best;
+        p.node = q.node;
+    }
+}
+
+// Sum over a warp, then over the block's warps in shared memory; thread 0 holds
+// the result.  wide: this thread's FP64 members are not all zero.
+__device__ __forceinline__ void diag_block_merge(DiagPartial& p, DiagPartial* sh, bool wide) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (__any_sync(FULL, wide)) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p.s[k] = warp_sum(p.s[k]);
+        p.bad = warp_sum(p.bad);
+        p.fast = warp_max(p.fast);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Two b;
+        b.hi = __shfl_down_sync(FULL, p.best.hi, o);
+        b.lo = __shfl_down_sync(FULL, p.best.lo, o);
+        const long long n = __shfl_down_sync(FULL, p.node, o);
+        if (n >= 0 && (p.node < 0 || two_less(p.best, b))) {
+            p.best = b;
+            p.node = n;
+        }
+    }
+    if (lane == 0) sh[wid] = p;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < DIAG_BLOCK / 32; ++w) diag_merge(p, sh[w]);
+}
+
+// out[0..5] as lb_diagnostics; out[6], out[7], out[8]: the error words of the
+// collision lists, the overlapped schedule and the TMA variant.
+template <class S>
+__global__ void __launch_bounds__(DIAG_BLOCK, 4) k_diagnostics(const __grid_constant__ LatticeArgs a, int c,
+                                                             DiagPartial* partials, unsigned* done,
+                                                             const int* rep_err, const int* sched_err, double* out) {
+    __shared__ DiagPartial sh[DIAG_BLOCK / 32];
+    __shared__ bool last;
     const ChannelDev& C = chan(a, c);
     const S* hs = (const S*)(a.par ? a.h1 : a.h0);
-    const uint8_t* fl = a.par ? a.fl0 : a.fl1;
-    const float4* gg = a.par ? a.g0 : a.g1;
-    double acc[DIAG_N] = {0, 0, 0, 0, 0, 0};
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < C.n; p += gridDim.x * blockDim.x) {
-        const long long gp = C.base + p;
+    DiagPartial p = {};
+    p.node = -1;
+    long long fs[4] = {0, 0, 0, 0};   // rho - 1 and momentum, 2^-56
+    int count = 0, pend = 0;
+    bool wide = false;                // this thread's part in FP64 is not empty
+    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < (unsigned)C.n; q += gridDim.x * blockDim.x) {
+        const long long gp = C.base + q;
         if (solid_at(a.mask, gp)) continue;
-        float h[Q];
-        int bad = 0;
+        float h[Q], drho, jx, jy, jz;
+        diag_moments<S>(a, hs, gp, h, drho, jx, jy, jz);
+        const bool small = fabsf(drho) < 1.0f && fabsf(jx) < 1.0f && fabsf(jy) < 1.0f && fabsf(jz) < 1.0f;
+        if (small) {
+            fs[0] += diag_fixed(drho);
+            fs[1] += diag_fixed(jx);
+            fs[2] += diag_fixed(jy);
+            fs[3] += diag_fixed(jz);
+            ++count;
+            if (++pend == 64) {   // |sums| < 64 2^56: no overflow before
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            h[i] = Pop<S>::ld(hs, (long long)i * a.Ntot + gp, i);
-            bad += !isfinite(h[i]);
+                for (int k = 0; k < 4; ++k) {
+                    p.s[k] += (double)fs[k] * 0x1p-56;
+                    fs[k] = 0;
+                }
+                pend = 0;
+                wide = true;
+            }
+        } else {
+            wide = true;
+            p.s[0] += 1.0 + (double)drho;
+            p.s[1] += jx; p.s[2] += jy; p.s[3] += jz;
+            if (!isfinite(drho))   // (a finite sum has finite terms)
+#pragma unroll
+                for (int i = 0; i < Q; ++i) p.bad += !isfinite(h[i]);
         }
-        float drho, jx, jy, jz;
-        moments(h, drho, jx, jy, jz);
-        acc[0] += 1.0 + (double)drho;
-        acc[1] += jx; acc[2] += jy; acc[3] += jz;
-        acc[4] += bad;
         if (a.has_last) {
-            float gx = C.G[0], gy = C.G[1], gz = C.G[2];
-            if (fl[gp >> 5]) { const float4 g = gg[gp]; gx += g.x; gy += g.y; gz += g.z; }
-            const double rho = 1.0 + (double)drho;
-            const double ux = (jx - 0.5 * gx) / rho, uy = (jy - 0.5 * gy) / rho, uz = (jz - 0.5 * gz) / rho;
-            const double um = sqrt(ux * ux + uy * uy + uz * uz);
-            acc[5] = (um != um) ? INFINITY : fmax(acc[5], um);
+            float gx, gy, gz;
+            diag_force(a, C, gp, gx, gy, gz);
+            const float vx = jx - 0.5f * gx, vy = jy - 0.5f * gy, vz = jz - 0.5f * gz;
+            const float rho = 1.0f + drho;
+            const float v2 = vx * vx + vy * vy + vz * vz;
+            if (small && rho > 0.01f && v2 > 1e-25f && v2 < 1e3f) {
+                // an upper bound of the node's |v|^2 / rho^2 (each component with
+                // more than its FP32 rounding error) decides whether it is compared
+                const float bx = fabsf(vx) + 1e-6f * (fabsf(jx) + fabsf(gx));
+                const float by = fabsf(vy) + 1e-6f * (fabsf(jy) + fabsf(gy));
+                const float bz = fabsf(vz) + 1e-6f * (fabsf(jz) + fabsf(gz));
+                if (__fdividef(bx * bx + by * by + bz * bz, rho * rho) * 1.0001f >= p.best.hi) {
+                    const Two x = two_sqr(two_sum(jx, -0.5f * gx)), y = two_sqr(two_sum(jy, -0.5f * gy)),
+                              z = two_sqr(two_sum(jz, -0.5f * gz));
+                    const Two w = two_div(two_add(two_add(x, y), z), two_sqr(two_sum(1.0f, drho)));
+                    if (p.node < 0 || two_less(p.best, w)) {
+                        p.best = w;
+                        p.node = gp;
+                    }
+                }
+            } else {
+                p.fast = fmax(p.fast, diag_speed(drho, jx, jy, jz, gx, gy, gz));
+                wide = true;
+            }
         }
     }
-    __shared__ double sh[DIAG_BLOCK / 32][DIAG_N];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // the block's integer sums, in two parts so that 256 of them cannot overflow
+    long long part[9];
 #pragma unroll
-    for (int k = 0; k < DIAG_N; ++k) {
-        const double v = (k == 5) ? warp_max(acc[k]) : warp_sum(acc[k]);
-        if (lane == 0) sh[wid][k] = v;
+    for (int k = 0; k < 4; ++k) {
+        part[2 * k] = fs[k] >> 28;
+        part[2 * k + 1] = fs[k] & 0xFFFFFFF;
+    }
+    part[8] = count;
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part[k] += __shfl_down_sync(FULL, part[k], o);
+    __shared__ long long shi[DIAG_BLOCK / 32][9];
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < 9; ++k) shi[threadIdx.x >> 5][k] = part[k];
+    diag_block_merge(p, sh, wide);
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < 9; ++k)
+            for (int w = 1; w < DIAG_BLOCK / 32; ++w) part[k] += shi[w][k];
+        for (int k = 0; k < 4; ++k) p.s[k] += (double)part[2 * k] * 0x1p-28 + (double)part[2 * k + 1] * 0x1p-56;
+        p.s[0] += (double)part[8];
+        partials[blockIdx.x] = p;
+        __threadfence();
+        last = atomicAdd(done, 1u) + 1 == gridDim.x;
     }
     __syncthreads();
-    if (threadIdx.x < DIAG_N) {
-        const int k = threadIdx.x;
-        double v = sh[0][k];
-        for (int w = 1; w < DIAG_BLOCK / 32; ++w) v = (k == 5) ? fmax(v, sh[w][k]) : v + sh[w][k];
-        partials[(long long)blockIdx.x * DIAG_N + k] = v;
+    if (!last) return;
+    __threadfence();
+    DiagPartial t = {};
+    t.node = -1;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += DIAG_BLOCK) diag_merge(t, partials[b]);
+    __syncthreads();
+    diag_block_merge(t, sh, true);
+    if (threadIdx.x == 0) {
+        if (t.node >= 0) {
+            float h[Q], drho, jx, jy, jz, gx, gy, gz;
+            diag_moments<S>(a, hs, t.node, h, drho, jx, jy, jz);
+            diag_force(a, C, t.node, gx, gy, gz);
+            t.fast = fmax(t.fast, diag_speed(drho, jx, jy, jz, gx, gy, gz));
+        }
+        for (int k = 0; k < 4; ++k) out[k] = t.s[k];
+        out[4] = t.bad;
+        out[5] = t.fast;
+        out[6] = rep_err ? (double)*rep_err : 0.0;
+        out[7] = (double)sched_err[0];
+        out[8] = (double)sched_err[1];
+        *done = 0u;
     }
 }
 
-__global__ void k_diag_final(const double* partials, int n_blocks, double* out) {
-    const int k = threadIdx.x;
-    if (k >= DIAG_N) return;
-    double v = 0.0;
-    for (int b = 0; b < n_blocks; ++b) {
-        const double x = partials[(long long)b * DIAG_N + k];
-        v = (k == 5) ? fmax(v, x) : v + x;
-    }
-    out[k] = v;
-}
+size_t diag_partial_bytes(int blocks) { return sizeof(DiagPartial) * (size_t)blocks; }
 
-cudaError_t launch_diagnostics(const LatticeArgs& a, int c, double* partials, int n_blocks, double* out,
-                               cudaStream_t s) {
-    if (a.storage == 0) k_diag_partial<float><<<n_blocks, DIAG_BLOCK, 0, s>>>(a, c, partials);
-    else if (a.storage == 1) k_diag_partial<__half><<<n_blocks, DIAG_BLOCK, 0, s>>>(a, c, partials);
-    else k_diag_partial<__nv_bfloat16><<<n_blocks, DIAG_BLOCK, 0, s>>>(a, c, partials);
-    k_diag_final<<<1, 32, 0, s>>>(partials, n_blocks, out);
+cudaError_t launch_diagnostics(const LatticeArgs& a, int c, int n, void* partials, int max_blocks, unsigned* done,
+                               const int* rep_err, const int* sched_err, double* out, cudaStream_t s) {
+    const int blocks = std::min(max_blocks, (n + DIAG_BLOCK - 1) / DIAG_BLOCK);
+    DiagPartial* p = (DiagPartial*)partials;
+    if (a.storage == 0) k_diagnostics<float><<<blocks, DIAG_BLOCK, 0, s>>>(a, c, p, done, rep_err, sched_err, out);
+    else if (a.storage == 1) k_diagnostics<__half><<<blocks, DIAG_BLOCK, 0, s>>>(a, c, p, done, rep_err, sched_err, out);
+    else k_diagnostics<__nv_bfloat16><<<blocks, DIAG_BLOCK, 0, s>>>(a, c, p, done, rep_err, sched_err, out);
     return cudaGetLastError();
 }
 

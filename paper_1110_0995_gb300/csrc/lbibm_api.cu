@@ -93,8 +93,10 @@ struct lb_ctx {
     uint8_t* fl[2] = {nullptr, nullptr};
     float4* u = nullptr;
     ChannelDev* d_ch = nullptr;
-    double* diag_partials = nullptr;
-    double* diag_out = nullptr;
+    char* diag_partials = nullptr;
+    double* diag_out = nullptr;      // [9], page-locked host memory that the kernel writes: the sums of
+                                     // lb_diagnostics and the error words
+    unsigned* diag_done = nullptr;
     int diag_blocks = 0;
     // immersed boundary, host staging
     std::vector<Q4> hq0, hq;
@@ -1100,9 +1102,11 @@ lb_status lb_create_batch(const lb_params* params, int n_channels, void* cuda_st
     TRY(dalloc(ctx, &ctx->dcount, 2));
     TRY(dalloc(ctx, &ctx->sched_err, 2));
     TRY(dalloc(ctx, &ctx->d_ch, ctx->ch.size()));
-    ctx->diag_blocks = 152 * 4;
-    TRY(dalloc(ctx, &ctx->diag_partials, (size_t)ctx->diag_blocks * 6));
-    TRY(dalloc(ctx, &ctx->diag_out, 6));
+    ctx->diag_blocks = ctx->sm_count * 4;
+    TRY(dalloc(ctx, &ctx->diag_partials, diag_partial_bytes(ctx->diag_blocks)));
+    TRY(cudaMallocHost((void**)&ctx->diag_out, 9 * sizeof(double)));
+    TRY(dalloc(ctx, &ctx->diag_done, 1));
+    TRY(cudaMemsetAsync(ctx->diag_done, 0, sizeof(unsigned), ctx->stream));
     TRY(cudaMemsetAsync(ctx->h[0], 0, (size_t)Q * ctx->plane * pop_bytes(ctx->storage), ctx->stream));
     TRY(cudaMemsetAsync(ctx->h[1], 0, (size_t)Q * ctx->plane * pop_bytes(ctx->storage), ctx->stream));
     TRY(cudaMemsetAsync(ctx->mask, 0, NG * 4, ctx->stream));
@@ -1178,6 +1182,7 @@ lb_status lb_destroy(lb_ctx* ctx) {
     for (auto& kv : ctx->adj.g_bwd) cudaGraphExecDestroy(kv.second);
     for (void* p : ctx->allocations) cudaFree(p);
     if (ctx->hq_pinned) cudaFreeHost(ctx->hq_pinned);
+    if (ctx->diag_out) cudaFreeHost(ctx->diag_out);
     ctx->allocations.clear();
     for (auto& ep : ctx->pending) { cudaEventDestroy(ep.a); cudaEventDestroy(ep.b); }
     for (auto e : ctx->free_events) cudaEventDestroy(e);
@@ -2392,21 +2397,16 @@ lb_status lb_diagnostics(lb_ctx* ctx, double u_max, double out[6]) {
     LB_GUARD(ctx);
     if (!out) return LB_ERR_ARG;
     const ChannelHost& c = ctx->ch[ctx->cur];
-    LB_CUDA(launch_diagnostics(lattice_args(ctx, (int)(ctx->step & 1)), ctx->cur, ctx->diag_partials,
-                               ctx->diag_blocks, ctx->diag_out, ctx->stream));
-    LB_CUDA(cudaMemcpyAsync(out, ctx->diag_out, sizeof(double) * 6, cudaMemcpyDeviceToHost, ctx->stream));
+    const double* res = ctx->diag_out;
+    LB_CUDA(launch_diagnostics(lattice_args(ctx, (int)(ctx->step & 1)), ctx->cur, c.d.n, ctx->diag_partials,
+                               ctx->diag_blocks, ctx->diag_done, ctx->rep_err, ctx->sched_err, ctx->diag_out, ctx->stream));
     LB_CUDA(cudaStreamSynchronize(ctx->stream));
+    std::copy(res, res + 6, out);
     if (out[4] > 0) return fail(ctx, LB_ERR_NUMERIC, "non-finite populations");
-    int serr = 0;
-    if (ctx->rep_err) {
-        LB_CUDA(cudaMemcpy(&serr, ctx->rep_err, sizeof(int), cudaMemcpyDeviceToHost));
-        if (serr > 0) return fail(ctx, LB_ERR_STATE, "collision candidate lists overflowed (more than 32 neighbour cells or 256 beads)");
-    }
-    int serr2[2] = {0, 0};
-    LB_CUDA(cudaMemcpy(serr2, ctx->sched_err, 2 * sizeof(int), cudaMemcpyDeviceToHost));
-    if (serr2[0] > 0)
+    if (res[6] > 0) return fail(ctx, LB_ERR_STATE, "collision candidate lists overflowed (more than 32 neighbour cells or 256 beads)");
+    if (res[7] > 0)
         return fail(ctx, LB_ERR_NUMERIC, "an IB point moved a lattice unit or more in one step (overlapped schedule)");
-    if (serr2[1] > 0) return fail(ctx, LB_ERR_TIMEOUT, "a TMA-staged stream-collide block gave up waiting for its copies");
+    if (res[8] > 0) return fail(ctx, LB_ERR_TIMEOUT, "a TMA-staged stream-collide block gave up waiting for its copies");
     if (u_max > 0 && !(out[5] <= u_max)) return fail(ctx, LB_ERR_NUMERIC, "velocity above the stability bound");
     return LB_OK;
 }

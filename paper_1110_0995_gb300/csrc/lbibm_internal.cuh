@@ -375,8 +375,11 @@ const void* stream_collide_bulk_func(int storage, int bs);
 cudaError_t prepare_bulk(int storage, int max_smem);   // allow up to max_smem dynamic bytes per bulk block
 cudaError_t launch_fields(const LatticeArgs& a, int ch_index, float* rho, float* u, cudaStream_t s);
 cudaError_t launch_pull_populations(const LatticeArgs& a, int ch_index, float* h_out, cudaStream_t s);
-cudaError_t launch_diagnostics(const LatticeArgs& a, int ch_index, double* partials, int n_blocks, double* out,
-                               cudaStream_t s);
+// n: nodes of the channel; partials: diag_partial_bytes(max_blocks); done: a zeroed
+// counter, left at zero; out: the six sums of lb_diagnostics and three error words
+size_t diag_partial_bytes(int blocks);
+cudaError_t launch_diagnostics(const LatticeArgs& a, int ch_index, int n, void* partials, int max_blocks, unsigned* done,
+                               const int* rep_err, const int* sched_err, double* out, cudaStream_t s);
 
 cudaError_t launch_cell_sums(const IbmArgs& a, cudaStream_t s);
 cudaError_t launch_elements(const IbmArgs& a, cudaStream_t s);
