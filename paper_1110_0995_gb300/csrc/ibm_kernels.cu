@@ -1,17 +1,13 @@
 // Immersed-boundary kernels (Gusenbauer et al., arXiv:1110.0995, Sec. 2.2-2.3):
 //   k_cell_sums      per-cell change of surface area and volume, FP32 per-triangle
 //                    terms added as exact 2^-40 fixed-point integers (Sec. 2.3.3:
-//                    the global area and volume constraints need every node of a cell)
-//   k_elements       the same per-triangle pass plus each triangle's area and
-//                    volume force terms, and per edge its stretching and
-//                    bending forces (Sec. 2.3.1), every element evaluated once
-//   k_forces_spread  node forces gathered from the element outputs of the
-//                    node's ring (deterministic order, no force atomics), then
-//                    spread with the trilinear delta function (Sec. 2.2 step 3)
+//                    the global area and volume constraints need every node of a
+//                    cell); the query's pass, the cycle's is in membrane.cu
+//   k_forces_spread  node forces from the membrane kernel's per-node sums and the
+//                    cell's global terms, spread with the trilinear delta
+//                    function (Sec. 2.2 step 3)
 //   k_interp_advance trilinear velocity interpolation (Sec. 2.2 step 1) and the
 //                    point advance X <- X + U (massless points)
-// The force kernel gives each IB node eight lanes: one ring slot and one
-// stencil corner per lane, so every load of a node is in flight at once.
 //
 // Positions are 64-bit fixed point (2^-40 lu); element geometry is FP32 formed
 // from exact fixed-point differences (see Pt below).
@@ -98,51 +94,6 @@ __device__ __forceinline__ const ChannelDev& chan(const IbmArgs& a, int c) {
 // division; every argument is positive for a non-degenerate element).
 __device__ __forceinline__ float sqrt_fast(float x) { return x * rsqrtf(x); }
 
-// Stretching (neo-Hookean bond, Dupin et al.): tension ks kappa(lambda)(lambda-1)
-// with kappa = (lambda^1/2 + lambda^-5/2)/(lambda + lambda^-3)
-//            = lambda^1/2 (lambda^3 + 1)/(lambda^4 + 1);
-// returns the force on a (the force on b is its negative).  a < b in global index.
-__device__ __forceinline__ float3 stretch_on_a(const Pt& A, const Pt& B, float L0, float ks) {
-    const float3 d = edge(A, B);
-    const float3 de = ddisp(A, B);
-    const float3 d0 = d - de;
-    const float num = 2.0f * dot(d0, de) + dot(de, de);   // |d|^2 - |d0|^2
-    const float L = sqrt_fast(L0 * L0 + num);
-    const float lm1 = __fdividef(num, (L + L0) * L0);      // lambda - 1
-    const float lam = 1.0f + lm1;
-    const float lam2 = lam * lam;
-    const float kappa = __fdividef(sqrt_fast(lam) * (lam2 * lam + 1.0f), lam2 * lam2 + 1.0f);
-    const float T = ks * kappa * lm1;
-    return (T * rsqrtf(dot(d, d))) * d;
-}
-
-// Bending: E = (kb/2)(theta - theta0)^2 at edge (a, b) between triangle (a, b, c)
-// and triangle (b, a, d); theta = atan2((n1 x n2).e_hat, n1.n2).  Writes the
-// forces on a, b, c, d (they sum to zero up to rounding).
-__device__ __forceinline__ void bend_all(const Pt& A, const Pt& B, const Pt& Cc, const Pt& D, float th0,
-                                         float kb, float3 f[4]) {
-    const float3 e = edge(A, B);
-    const float3 ac = edge(A, Cc);
-    const float3 ad = edge(A, D);
-    const float3 bd = ad - e;
-    const float3 n1 = cross(e, ac);
-    const float3 n2 = cross(-e, bd);
-    const float l2 = dot(e, e);
-    const float rl = rsqrtf(l2);
-    const float l = l2 * rl;
-    const float theta = atan2f(dot(cross(n1, n2), e) * rl, dot(n1, n2));
-    const float coef = -kb * (theta - th0);
-    const float3 gc = __fdividef(-l, dot(n1, n1)) * n1;
-    const float3 gd = __fdividef(-l, dot(n2, n2)) * n2;
-    const float il2 = __fdividef(1.0f, l2);
-    const float sc = dot(ac, e) * il2;
-    const float sd = dot(ad, e) * il2;
-    f[0] = coef * ((-(1.0f - sc)) * gc - (1.0f - sd) * gd);
-    f[1] = coef * ((-sc) * gc - sd * gd);
-    f[2] = coef * gc;
-    f[3] = coef * gd;
-}
-
 // Area change of triangle (0, 1, 2) from rest: S_t - S0_t from
 // |n|^2 - |n0|^2 = 2 n0.dn + dn.dn, dn = a1 x b2 + b1 x a2 + b1 x b2.
 __device__ __forceinline__ float tri_dS(const float3& e1, const float3& e2, const float3& b1, const float3& b2,
@@ -173,13 +124,8 @@ __device__ __forceinline__ float tri_dV6(const Pt& R, const Pt& P0, const Pt& P1
 // units (each rounded once, far below its FP32 rounding; the sums are exact
 // and independent of their order, and run on the integer pipe: this GPU's
 // FP64 pipe retires about two operations per clock per SM).  The last block
-// of a cell adds the cell's partials and forms dS, dV in FP64 once.  With
-// FORCES the same pass
-// writes each triangle's area and volume force terms:
-//   area (local + global, homocentric): F_k = (kal dS_t/S0_t + kag dS/S0) a_k,
-//     a_k = -(2 S_t / sum_j |w_j|^2) w_k, w_k = x_k - centroid;
-//   volume: F_k = -kv (dV/V0) n_t / 6, n_t = (x_1 - x_0) x (x_2 - x_0).
-// The cell totals dS/S0 and dV/V0 are applied in the node gather.
+// of a cell adds the cell's partials and forms dS, dV in FP64 once.
+// ---------------------------------------------------------------------------
 // ---------------------------------------------------------------------------
 // Block size and register budget of the immersed-boundary kernels: 128
 // threads within 64 registers (8192 per block), so that one such block fits
@@ -234,113 +180,24 @@ __device__ __forceinline__ void chunk_sums(const IbmArgs& a, int chunk, const in
     }
 }
 
-// The static data of one triangle (indices, rest area, the cell's reference
-// node and local-area modulus), which the element pass loads before waiting
-// for the previous advance.
-struct TriStatic {
-    int4 tr;
-    float S0t, kal;
-    int ref;
-};
-
-__device__ __forceinline__ TriStatic tri_static(const IbmArgs& a, int t) {
-    TriStatic d;
-    d.tr = a.tris[t];
-    d.S0t = a.tri_S0[t];
-    d.ref = a.cells[d.tr.w].ref;
-    d.kal = a.cells[d.tr.w].kal;
-    return d;
-}
-
-// dS_t and dV_t (x 6) of one triangle; with FORCES also its area and volume
-// force terms.
-template <bool FORCES>
-__device__ __forceinline__ void tri_terms(const IbmArgs& a, int t, const TriStatic& d, long long& s, long long& v) {
-    const Q4* qc = cur_q(a);
-    const Pt R = load_pt(a, qc, d.ref);
-    const Pt P0 = load_pt(a, qc, d.tr.x), P1 = load_pt(a, qc, d.tr.y), P2 = load_pt(a, qc, d.tr.z);
-    const float3 e1 = edge(P0, P1), e2 = edge(P0, P2);
-    const float dSt = tri_dS(e1, e2, ddisp(P0, P1), ddisp(P0, P2), d.S0t);
-    s += float_to_fixed(dSt);
-    v += float_to_fixed(tri_dV6(R, P0, P1, P2));
-    if constexpr (FORCES) {
-        const float St = d.S0t + dSt;
-        const float3 third = (1.0f / 3.0f) * (e1 + e2);
-        const float3 w0 = -third, w1 = e1 - third, w2 = e2 - third;
-        const float ww = dot(w0, w0) + dot(w1, w1) + dot(w2, w2);
-        const float c = __fdividef(-2.0f * St, ww);
-        const float sl = __fdividef(d.kal * dSt, d.S0t);
-        a.tA[3 * t] = make_float4(c * w0.x, c * w0.y, c * w0.z, sl);
-        a.tA[3 * t + 1] = make_float4(c * w1.x, c * w1.y, c * w1.z, sl);
-        a.tA[3 * t + 2] = make_float4(c * w2.x, c * w2.y, c * w2.z, sl);
-        const float3 n = cross(e1, e2);
-        a.tN[t] = make_float4(n.x, n.y, n.z, 0.f);
-    }
-}
-
-template <bool FORCES>
-__device__ __forceinline__ void tri_chunk(const IbmArgs& a, int chunk) {
-    const int4 ck = a.chunks[chunk];
-    long long s = 0, v = 0;
-    for (int t = ck.y + (int)threadIdx.x; t < ck.z; t += CS_BLOCK) tri_terms<FORCES>(a, t, tri_static(a, t), s, v);
-    chunk_sums(a, chunk, ck, s, v);
-}
-
 __global__ void __launch_bounds__(CS_BLOCK, 6) k_cell_sums(const __grid_constant__ IbmArgs a) {
-    tri_chunk<false>(a, blockIdx.x);
+    const int4 ck = a.chunks[blockIdx.x];
+    const Q4* qc = cur_q(a);
+    long long s = 0, v = 0;
+    for (int t = ck.y + (int)threadIdx.x; t < ck.z; t += CS_BLOCK) {
+        const int4 tr = a.tris[t];
+        const Pt R = load_pt(a, qc, a.cells[tr.w].ref);
+        const Pt P0 = load_pt(a, qc, tr.x), P1 = load_pt(a, qc, tr.y), P2 = load_pt(a, qc, tr.z);
+        s += float_to_fixed(tri_dS(edge(P0, P1), edge(P0, P2), ddisp(P0, P1), ddisp(P0, P2), a.tri_S0[t]));
+        v += float_to_fixed(tri_dV6(R, P0, P1, P2));
+    }
+    chunk_sums(a, blockIdx.x, ck, s, v);
 }
 
 cudaError_t launch_cell_sums(const IbmArgs& a, cudaStream_t s) {
     if (a.n_chunks <= 0) return cudaSuccess;
     k_cell_sums<<<a.n_chunks, CS_BLOCK, 0, s>>>(a);
     return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Element pass: blocks [0, n_chunks) are the triangle chunks above (with their
-// force terms), the blocks after them take one edge per thread: stretching
-// (neo-Hookean bond) and bending of edge (a, b), each evaluated once.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(CS_BLOCK, 6) k_elements(const __grid_constant__ IbmArgs a) {
-    if ((int)blockIdx.x < a.n_chunks) {
-        // a chunk holds at most one triangle per thread: its static data
-        // before the previous advance has finished, then its positions
-        const int4 ck = a.chunks[blockIdx.x];
-        const int t = ck.y + (int)threadIdx.x;
-        const bool live = t < ck.z;
-        TriStatic d = {};
-        if (live) d = tri_static(a, t);
-        pdl_entry();
-        long long s = 0, v = 0;
-        if (live) tri_terms<true>(a, t, d, s, v);
-        chunk_sums(a, blockIdx.x, ck, s, v);
-        return;
-    }
-    // the edge's static data before the previous advance has finished
-    const int e = ((int)blockIdx.x - a.n_chunks) * CS_BLOCK + (int)threadIdx.x;
-    const bool live = e < a.n_edges;
-    int4 ev = make_int4(0, 0, 0, 0);
-    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);   // (L0, theta0, ks, kb)
-    if (live) {
-        ev = a.edges[e];
-        r = a.edge_rest[e];
-    }
-    pdl_entry();
-    if (!live) return;
-    const Q4* qc = cur_q(a);
-    const Pt A = load_pt(a, qc, ev.x), B = load_pt(a, qc, ev.y), Cc = load_pt(a, qc, ev.z), D = load_pt(a, qc, ev.w);
-    const float3 fs = stretch_on_a(A, B, r.x, r.z);
-    a.eS[e] = make_float4(fs.x, fs.y, fs.z, 0.f);
-    float3 fb[4];
-    bend_all(A, B, Cc, D, r.y, r.w, fb);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) a.eB[4 * e + k] = make_float4(fb[k].x, fb[k].y, fb[k].z, 0.f);
-}
-
-cudaError_t launch_elements(const IbmArgs& a, cudaStream_t s) {
-    const int blocks = a.n_chunks + (a.n_edges + CS_BLOCK - 1) / CS_BLOCK;
-    if (blocks <= 0) return cudaSuccess;
-    return launch_ex(k_elements, blocks, CS_BLOCK, 0, s, a.pdl, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -443,12 +300,29 @@ cudaError_t launch_compact_groups(const uint8_t* map, int n_groups, int* list, i
 }
 
 // ---------------------------------------------------------------------------
-// node forces + spreading, eight lanes per IB node: each lane gathers the
-// node's share of the elements of some ring slots (incident triangle, edge and
-// opposite edge; fixed order, no atomics), the eight partial sums are added by
-// shuffles, then each lane spreads to one stencil corner.
+// node forces + spreading, eight lanes per IB node: the node's membrane force
+// from the membrane kernel's sums and the cell's global terms, then each lane
+// spreads to one stencil corner.
 // ---------------------------------------------------------------------------
 constexpr int FS_BLOCK = 128;
+
+// The membrane force of node i: local part + kag (dS / S0) sum of area
+// directions - kv (dV / V0) / 6 sum of normals.
+__device__ __forceinline__ float3 node_force(const IbmArgs& a, int i, float kag, float kv, int cid) {
+    const float2 rel = a.cell_rel[cid];
+    const float4 p = a.acc[3 * (size_t)i], q = a.acc[3 * (size_t)i + 1];
+    const float nz = a.acc[3 * (size_t)i + 2].x;
+    const float kag_dS = kag * rel.x;
+    const float kv_dV6 = kv * rel.y * (1.0f / 6.0f);
+    float3 F = make_float3(p.x + (kag_dS * p.w - kv_dV6 * q.z), p.y + (kag_dS * q.x - kv_dV6 * q.w),
+                           p.z + (kag_dS * q.y - kv_dV6 * nz));
+    if (a.R) {
+        // collisions (Sec. 2.4)
+        const float4 r = a.R[i];
+        F.x += r.x; F.y += r.y; F.z += r.z;
+    }
+    return F;
+}
 
 #ifndef LBIBM_FS_MINB
 #define LBIBM_FS_MINB 10
@@ -459,19 +333,16 @@ __global__ void __launch_bounds__(FS_BLOCK, MASSIVE ? IB_MIN_BLOCKS : LBIBM_FS_M
     const int i = (blockIdx.x * FS_BLOCK + threadIdx.x) / SUB;
     const int sl = threadIdx.x & (SUB - 1);
     const bool live = i < a.n_nodes;
-    // before the element pass has finished: the node's static data, its
+    // before the membrane kernel has finished: the node's static data, its
     // position (advanced in the previous cycle) and this lane's stencil corner
     // (Sec. 2.2 step 3) with its obstacle bit
-    // and the lane's first ring slot
     int4 inf = make_int4(0, 0, 0, 0);
-    int4 sr0 = make_int4(0, 0, 0, 0);
     Q4 qi = {};
     long long g = 0;
     float w = 0.f;
     bool hit = false;
     if (live) {
         inf = a.info[i];
-        if (sl < (inf.w & 0xff)) sr0 = a.slots[inf.z + sl];
         qi = (a.par ? a.qb : a.qa)[i];
         hit = corner(chan(a, inf.w >> 8), qi, sl, g, w);
         if (hit) hit = !((__ldg(a.mask + (g >> 5)) >> (g & 31)) & 1u);
@@ -479,9 +350,8 @@ __global__ void __launch_bounds__(FS_BLOCK, MASSIVE ? IB_MIN_BLOCKS : LBIBM_FS_M
     pdl_entry();
     if (!live) return;   // whole groups of eight lanes leave together
     const unsigned smask = 0xffu << (threadIdx.x & 24);
-    const int cid = inf.x, k0 = inf.z, k = inf.w & 0xff, chn = inf.w >> 8;
+    const int cid = inf.x, chn = inf.w >> 8;
     const CellDev& C = a.cells[cid];
-    const float2 rel = a.cell_rel[cid];
     const ChannelDev Ch = chan(a, chn);
     if (a.dcur) {
         // overlapped schedule: the target must be in this step's stencil set
@@ -491,33 +361,7 @@ __global__ void __launch_bounds__(FS_BLOCK, MASSIVE ? IB_MIN_BLOCKS : LBIBM_FS_M
         mark_box(Ch, qi, sl, a.dmark);
     }
 
-    const float kag_dS = C.kag * rel.x;
-    const float kv_dV6 = C.kv * rel.y * (1.0f / 6.0f);
-    float3 F = make_float3(0.f, 0.f, 0.f);
-    for (int s = sl; s < k; s += SUB) {
-        const int4 sr = s == sl ? sr0 : a.slots[k0 + s];
-        const float4 ta = a.tA[sr.x];
-        const float4 tn = a.tN[sr.w];
-        const float4 es = a.eS[sr.y >> 2];
-        const float4 b1 = a.eB[sr.y];
-        const float4 b2 = a.eB[sr.z];
-        const float sg = (sr.y & 3) == 0 ? 1.0f : -1.0f;   // stretching acts on a, its negative on b
-        const float ca = ta.w + kag_dS;
-        F.x += ((ca * ta.x - kv_dV6 * tn.x) + sg * es.x) + (b1.x + b2.x);
-        F.y += ((ca * ta.y - kv_dV6 * tn.y) + sg * es.y) + (b1.y + b2.y);
-        F.z += ((ca * ta.z - kv_dV6 * tn.z) + sg * es.z) + (b1.z + b2.z);
-    }
-#pragma unroll
-    for (int o = SUB / 2; o > 0; o >>= 1) {
-        F.x += __shfl_xor_sync(smask, F.x, o);
-        F.y += __shfl_xor_sync(smask, F.y, o);
-        F.z += __shfl_xor_sync(smask, F.z, o);
-    }
-    if (a.R) {
-        // collisions (Sec. 2.4): every lane holds the reduced total, add to each
-        const float4 r = a.R[i];
-        F.x += r.x; F.y += r.y; F.z += r.z;
-    }
+    const float3 F = node_force(a, i, C.kag, C.kv, cid);
     if (sl == 0) a.F[i] = make_float4(F.x, F.y, F.z, 0.f);
 
     uint8_t* fl = a.par ? a.fl1 : a.fl0;
@@ -576,8 +420,8 @@ __global__ void __launch_bounds__(FS_BLOCK, MASSIVE ? IB_MIN_BLOCKS : LBIBM_FS_M
     if (hit && (__ffs(same) - 1) == (int)(threadIdx.x & 31)) fl[grp] = 1;
 }
 
-// The massless node forces + spreading with four lanes per IB node (each
-// lane two ring slots and two stencil corners): half the threads of the
+// The massless node forces + spreading with four lanes per IB node (two
+// stencil corners each): half the threads of the
 // eight-lane kernel for the sequential schedule (the overlapped schedule's
 // stencil marking and points with mass keep eight lanes).
 constexpr int FS4 = 4;
@@ -586,19 +430,18 @@ __global__ void __launch_bounds__(FS_BLOCK, 9) k_forces_spread4(const __grid_con
     const int i = (blockIdx.x * FS_BLOCK + threadIdx.x) / FS4;
     const int sl = threadIdx.x & (FS4 - 1);
     const bool live = i < a.n_nodes;
-    // before the element pass has finished: the node's static data, its
-    // position (advanced in the previous cycle), this lane's two stencil
-    // corners with their obstacle bits and its first two ring slots
+    // before the membrane kernel has finished: the node's static data, its
+    // position (advanced in the previous cycle) and this lane's two stencil
+    // corners with their obstacle bits
     int4 inf = make_int4(0, 0, 0, 0);
-    int4 sr0 = make_int4(0, 0, 0, 0), sr1 = make_int4(0, 0, 0, 0);
+    float kag = 0.f, kv = 0.f;
     long long g[2] = {0, 0};
     float w[2] = {0.f, 0.f};
     bool hit[2] = {false, false};
     if (live) {
         inf = a.info[i];
-        const int k = inf.w & 0xff;
-        if (sl < k) sr0 = a.slots[inf.z + sl];
-        if (sl + FS4 < k) sr1 = a.slots[inf.z + sl + FS4];
+        kag = a.cells[inf.x].kag;
+        kv = a.cells[inf.x].kv;
         const Q4 qi = (a.par ? a.qb : a.qa)[i];
         const ChannelDev& Ch = chan(a, inf.w >> 8);
 #pragma unroll
@@ -609,36 +452,7 @@ __global__ void __launch_bounds__(FS_BLOCK, 9) k_forces_spread4(const __grid_con
     }
     pdl_entry();
     if (!live) return;   // whole groups of four lanes leave together
-    const unsigned smask = 0xfu << (threadIdx.x & 28);
-    const int cid = inf.x, k0 = inf.z, k = inf.w & 0xff;
-    const CellDev& C = a.cells[cid];
-    const float2 rel = a.cell_rel[cid];
-    const float kag_dS = C.kag * rel.x;
-    const float kv_dV6 = C.kv * rel.y * (1.0f / 6.0f);
-    float3 F = make_float3(0.f, 0.f, 0.f);
-    for (int s = sl; s < k; s += FS4) {
-        const int4 sr = s == sl ? sr0 : (s == sl + FS4 ? sr1 : a.slots[k0 + s]);
-        const float4 ta = a.tA[sr.x];
-        const float4 tn = a.tN[sr.w];
-        const float4 es = a.eS[sr.y >> 2];
-        const float4 b1 = a.eB[sr.y];
-        const float4 b2 = a.eB[sr.z];
-        const float sg = (sr.y & 3) == 0 ? 1.0f : -1.0f;   // stretching acts on a, its negative on b
-        const float ca = ta.w + kag_dS;
-        F.x += ((ca * ta.x - kv_dV6 * tn.x) + sg * es.x) + (b1.x + b2.x);
-        F.y += ((ca * ta.y - kv_dV6 * tn.y) + sg * es.y) + (b1.y + b2.y);
-        F.z += ((ca * ta.z - kv_dV6 * tn.z) + sg * es.z) + (b1.z + b2.z);
-    }
-#pragma unroll
-    for (int o = FS4 / 2; o > 0; o >>= 1) {
-        F.x += __shfl_xor_sync(smask, F.x, o);
-        F.y += __shfl_xor_sync(smask, F.y, o);
-        F.z += __shfl_xor_sync(smask, F.z, o);
-    }
-    if (a.R) {
-        const float4 r = a.R[i];
-        F.x += r.x; F.y += r.y; F.z += r.z;
-    }
+    const float3 F = node_force(a, i, kag, kv, inf.x);
     if (sl == 0) a.F[i] = make_float4(F.x, F.y, F.z, 0.f);
     uint8_t* fl = a.par ? a.fl1 : a.fl0;
     const unsigned active = __activemask();

@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <future>
 #include <map>
 #include <memory>
 #include <string>
@@ -54,13 +55,24 @@ struct MeshConn {
     std::vector<int4> edges;
     std::vector<int4> slots;
     std::vector<int> ring_off, valence;
+    // its patches, built on a host thread while the caller goes on adding
+    // meshes, and where the commit put them in the context's tables
+    std::future<PatchTables> patches;
+    int patch0 = -1, n_patch = 0;
 };
 
+PatchTables conn_patches(const MeshConn& c) {
+    PatchTables t;
+    build_patches(MeshTables{c.n, c.nt, (int)c.edges.size(), c.tris.data(), c.edges.data(), c.slots.data(),
+                             c.ring_off.data(), c.valence.data()}, t);
+    return t;
+}
+
 // A mesh added to the context: its connectivity and where its nodes,
-// triangles, edges and ring slots go in the context's tables.
+// triangles and edges go in the context's tables.
 struct PendingMesh {
-    const MeshConn* conn;
-    int node0, tri0, e0, slot0, cell, ch;
+    MeshConn* conn;
+    int node0, tri0, e0, cell, ch;
     float ks, kb;
 };
 
@@ -101,7 +113,6 @@ struct lb_ctx {
     // immersed boundary, host staging
     std::vector<Q4> hq0, hq;
     std::vector<int4> hinfo;
-    std::vector<int4> hslots;      // ring CSR: element outputs of each ring slot
     std::vector<int4> hedges;      // (a, b, c, d)
     std::vector<float4> hedge_rest;  // (L0, theta0, ks, kb)
     std::vector<int4> htris;
@@ -111,13 +122,13 @@ struct lb_ctx {
     std::vector<double> hrest;     // rest positions (x, y, z per node)
     std::vector<std::unique_ptr<MeshConn>> conn_cache;   // connectivity per distinct triangle list
     std::vector<PendingMesh> pending_meshes;             // meshes whose tables the commit writes
-    int n_tris_staged = 0, n_edges_staged = 0, n_slots_staged = 0;
+    int n_tris_staged = 0, n_edges_staged = 0;
     float* fields_buf = nullptr;   // device scratch of lb_get_fields (4 floats per node of the largest channel)
     std::vector<MeshHost> meshes;
     std::vector<std::vector<int>> ch_meshes;
     bool committed = false;
     // immersed boundary, device
-    int M = 0, C = 0, T = 0, NCH = 0, K = 0, E = 0;
+    int M = 0, C = 0, T = 0, NCH = 0, E = 0;
     Q4* q[2] = {nullptr, nullptr};
     Q4* q0 = nullptr;
     float4* F = nullptr;
@@ -125,10 +136,18 @@ struct lb_ctx {
     double* d_xyz = nullptr;       // [3M] device staging of asynchronous readbacks
     cudaEvent_t rb_ev[2] = {nullptr, nullptr};
     int4* info = nullptr;
-    int4* slots = nullptr;
     int4* edges = nullptr;
     float4* edge_rest = nullptr;
-    float4 *eS = nullptr, *eB = nullptr, *tA = nullptr, *tN = nullptr;
+    // membrane kernel: a job per block, the patches' tables, the node sums
+    int n_patches = 0;
+    size_t patch_smem = 0;
+    PatchJob* patches = nullptr;
+    uint32_t* ploc = nullptr;
+    uint2 *ptri = nullptr, *pedge = nullptr, *pring = nullptr;
+    float2* prest_edge = nullptr;
+    float* prest_tri = nullptr;
+    Fix3* prest_node = nullptr;
+    float4* acc = nullptr;
     int4* tris = nullptr;
     float* triS0 = nullptr;
     int4* chunks = nullptr;
@@ -373,14 +392,18 @@ IbmArgs ibm_args(const lb_ctx* ctx, int par, bool overlapped = false) {
     a.qa = ctx->q[0];
     a.qb = ctx->q[1];
     a.q0 = ctx->q0;
-    a.slots = ctx->slots;
-    a.edges = ctx->edges;
-    a.edge_rest = ctx->edge_rest;
-    a.n_edges = ctx->E;
-    a.eS = ctx->eS;
-    a.eB = ctx->eB;
-    a.tA = ctx->tA;
-    a.tN = ctx->tN;
+    a.patches = ctx->patches;
+    a.n_patches = ctx->n_patches;
+    a.patch_smem = (int)ctx->patch_smem;
+    a.ploc = ctx->ploc;
+    a.ptri = ctx->ptri;
+    a.pedge = ctx->pedge;
+    a.pring = ctx->pring;
+    a.prest_edge = ctx->prest_edge;
+    a.prest_tri = ctx->prest_tri;
+    a.prest_node = ctx->prest_node;
+    a.sm_count = ctx->sm_count;
+    a.acc = ctx->acc;
     a.F = ctx->F;
     a.tris = ctx->tris;
     a.tri_S0 = ctx->triS0;
@@ -506,7 +529,7 @@ lb_status enqueue_step(lb_ctx* ctx, int par) {
         }
         cudaError_t e = cudaSuccess;
         switch (k) {
-            case 0: e = launch_elements(ia, ctx->stream); break;
+            case 0: e = launch_membrane(ia, ctx->stream); break;
             case 1:
                 e = launch_forces_spread(ia, ctx->stream);
                 if (e == cudaSuccess && ia.gfix) e = launch_gfix_to_g(ia, ctx->stream);
@@ -584,7 +607,7 @@ lb_status enqueue_step_overlap(lb_ctx* ctx, int par, bool lead_interp) {
     LB_CUDA(cudaMemsetAsync(ctx->dcount + (1 - par), 0, sizeof(int), ib));
     cudaError_t e = cudaSuccess;
     if (lead_interp && e == cudaSuccess) e = launch_interp_advance(ibm_args(ctx, 1 - par), ib);
-    if (e == cudaSuccess) e = launch_elements(ia, ib);
+    if (e == cudaSuccess) e = launch_membrane(ia, ib);
     if (e == cudaSuccess) e = launch_forces_spread(ia, ib);
     if (e == cudaSuccess) e = launch_compact_groups(ctx->dmap[1 - par], (int)NG, ctx->dlist[1 - par], ctx->dcount + (1 - par), ib);
     if (e == cudaSuccess) e = launch_stream_collide_split(la, ctx->k3.bs, 1, ctx->total_blocks, bulk_smem(ctx), m);
@@ -801,17 +824,17 @@ void apply_k3_config(lb_ctx* ctx, K3Config c) {
 
 // The element and ring tables of every mesh (triangles with their rest
 // areas, edges with rest length and rest dihedral angle (the bending's
-// theta0, Sec. 2.3.1), each node's ring slots), written at the commit, the
+// theta0, Sec. 2.3.1)), written at the commit, the
 // meshes spread over up to 16 host threads (each writes only its own ranges).
-void build_tables(lb_ctx* ctx) {
+template <class After>
+void build_tables(lb_ctx* ctx, After after) {
     ctx->htris.resize(ctx->n_tris_staged);
     ctx->htriS0.resize(ctx->n_tris_staged);
     ctx->hedges.resize(ctx->n_edges_staged);
     ctx->hedge_rest.resize(ctx->n_edges_staged);
-    ctx->hslots.resize(ctx->n_slots_staged);
     ctx->hinfo.resize(ctx->hq0.size());
     const double* x = ctx->hrest.data();
-    auto one = [ctx, x](const PendingMesh& pm) {
+    auto one = [ctx, x, &after](const PendingMesh& pm) {
         const MeshConn& c = *pm.conn;
         const int node0 = pm.node0;
         for (int t = 0; t < c.nt; ++t) {
@@ -832,11 +855,8 @@ void build_tables(lb_ctx* ctx) {
             ctx->hedge_rest[pm.e0 + k] = make_float4((float)L0, (float)th0, pm.ks, pm.kb);
         }
         for (int i = 0; i < c.n; ++i)
-            ctx->hinfo[node0 + i] = make_int4(pm.cell, node0, pm.slot0 + c.ring_off[i], c.valence[i] | (pm.ch << 8));
-        for (size_t k = 0; k < c.slots.size(); ++k) {
-            const int4 sl = c.slots[k];
-            ctx->hslots[pm.slot0 + k] = make_int4(3 * pm.tri0 + sl.x, 4 * pm.e0 + sl.y, 4 * pm.e0 + sl.z, pm.tri0 + sl.w);
-        }
+            ctx->hinfo[node0 + i] = make_int4(pm.cell, node0, 0, pm.ch << 8);
+        after(pm);
     };
     const int nm = (int)ctx->pending_meshes.size();
     const int nth = std::max(1, std::min({16, (int)std::thread::hardware_concurrency(), nm / 4}));
@@ -860,15 +880,87 @@ void build_tables(lb_ctx* ctx) {
     ctx->pending_meshes.clear();
 }
 
-lb_status commit_ibm(lb_ctx* ctx) {
-    if (ctx->committed) return LB_OK;
-    ctx->committed = true;
-    build_tables(ctx);
+lb_status commit_tables(lb_ctx* ctx) {
+    // the patches of every distinct connectivity, then the cells' jobs on them
+    PatchTables ptabs;
+    std::vector<PatchJob> hpatches;
+    std::vector<int> cell_patch0(ctx->hcells.size(), 0);
+    int n_rest[3] = {0, 0, 0};
+    for (const PendingMesh& pm : ctx->pending_meshes) {
+        MeshConn& c = *pm.conn;
+        if (c.patch0 < 0) {
+            PatchTables t = c.patches.valid() ? c.patches.get() : conn_patches(c);
+            c.patch0 = (int)ptabs.tab.size();
+            c.n_patch = (int)t.tab.size();
+            for (PatchTab& p : t.tab) {
+                p.loc0 += (int)ptabs.loc.size();
+                p.tri0 += (int)ptabs.tri.size();
+                p.edge0 += (int)ptabs.edge.size();
+                p.ring0 += (int)ptabs.ring.size();
+            }
+            auto append = [](auto& to, const auto& from) { to.insert(to.end(), from.begin(), from.end()); };
+            append(ptabs.tab, t.tab);
+            append(ptabs.loc, t.loc);
+            append(ptabs.tri, t.tri);
+            append(ptabs.edge, t.edge);
+            append(ptabs.ring, t.ring);
+            append(ptabs.tri_id, t.tri_id);
+            append(ptabs.edge_id, t.edge_id);
+        }
+        // positions relative to the reference node split at 2^-grid: 16 where the
+        // cell reaches at most 64 lu from it, so that the upper parts (23 bits
+        // with room for twice the extent) and the lower ones are exact in FP32
+        const double* x = ctx->hrest.data() + 3 * (size_t)pm.node0;
+        double ext = 1.0;
+        for (int k = 0; k < 3 * c.n; ++k) ext = std::max(ext, std::fabs(x[k] - x[k % 3]));
+        const CellDev& cd = ctx->hcells[pm.cell];
+        PatchJob job = {};
+        job.cell = pm.cell;
+        job.ref = cd.ref;
+        job.node0 = pm.node0;
+        job.grid = std::max(0, std::min(16, 22 - (int)std::ceil(std::log2(ext))));
+        job.patch0 = cell_patch0[pm.cell] = (int)hpatches.size();
+        job.n_patch = c.n_patch;
+        job.ks = cd.ks;
+        job.kb = cd.kb;
+        job.kal = cd.kal;
+        for (int k = 0; k < c.n_patch; ++k) {
+            job.tab = ptabs.tab[c.patch0 + k];
+            job.rest_edge = n_rest[0];
+            job.rest_tri = n_rest[1];
+            job.rest_node = n_rest[2];
+            n_rest[0] += job.tab.n_edge;
+            n_rest[1] += job.tab.n_tri;
+            n_rest[2] += job.tab.n_loc;
+            hpatches.push_back(job);
+        }
+    }
+    ctx->n_patches = (int)hpatches.size();
+    for (const PatchTab& t : ptabs.tab) ctx->patch_smem = std::max(ctx->patch_smem, patch_smem_bytes(t));
+    std::vector<float2> rest_edge(n_rest[0]);
+    std::vector<float> rest_tri(n_rest[1]);
+    std::vector<Fix3> rest_node(n_rest[2]);
+    build_tables(ctx, [&](const PendingMesh& pm) {
+        // a cell's rest data in its patches' order
+        const CellDev& cd = ctx->hcells[pm.cell];
+        const Q4 r = ctx->hq0[cd.ref];
+        for (int b = cell_patch0[pm.cell], k = 0; k < pm.conn->n_patch; ++k, ++b) {
+            const PatchJob& j = hpatches[b];
+            for (int i = 0; i < j.tab.n_edge; ++i) {
+                const float4 e = ctx->hedge_rest[pm.e0 + ptabs.edge_id[j.tab.edge0 + i]];
+                rest_edge[j.rest_edge + i] = make_float2(e.x, e.y);
+            }
+            for (int i = 0; i < j.tab.n_tri; ++i) rest_tri[j.rest_tri + i] = ctx->htriS0[pm.tri0 + ptabs.tri_id[j.tab.tri0 + i]];
+            for (int i = 0; i < j.tab.n_loc; ++i) {
+                const Q4& q = ctx->hq0[pm.node0 + ptabs.loc[j.tab.loc0 + i]];
+                rest_node[j.rest_node + i] = Fix3{q.x - r.x, q.y - r.y, q.z - r.z};
+            }
+        }
+    });
     ctx->M = (int)ctx->hq0.size();
     ctx->C = (int)ctx->hcells.size();
     ctx->T = (int)ctx->htris.size();
     ctx->NCH = (int)ctx->hchunks.size();
-    ctx->K = (int)ctx->hslots.size();
     ctx->E = (int)ctx->hedges.size();
     if (ctx->M == 0) return LB_OK;
     auto up = [&](auto** dst, const auto& src) -> cudaError_t {
@@ -881,7 +973,6 @@ lb_status commit_ibm(lb_ctx* ctx) {
     LB_CUDA(up(&ctx->q[0], ctx->hq));
     LB_CUDA(up(&ctx->q[1], ctx->hq));
     LB_CUDA(up(&ctx->info, ctx->hinfo));
-    LB_CUDA(up(&ctx->slots, ctx->hslots));
     if (ctx->rep_k > 0.f) {
         std::vector<Q4> bq;
         std::vector<float> br;
@@ -915,10 +1006,15 @@ lb_status commit_ibm(lb_ctx* ctx) {
     }
     LB_CUDA(up(&ctx->edges, ctx->hedges));
     LB_CUDA(up(&ctx->edge_rest, ctx->hedge_rest));
-    LB_CUDA(dalloc(ctx, &ctx->eS, ctx->E));
-    LB_CUDA(dalloc(ctx, &ctx->eB, 4 * (size_t)ctx->E));
-    LB_CUDA(dalloc(ctx, &ctx->tA, 3 * (size_t)ctx->T));
-    LB_CUDA(dalloc(ctx, &ctx->tN, ctx->T));
+    LB_CUDA(up(&ctx->patches, hpatches));
+    LB_CUDA(up(&ctx->ploc, ptabs.loc));
+    LB_CUDA(up(&ctx->ptri, ptabs.tri));
+    LB_CUDA(up(&ctx->pedge, ptabs.edge));
+    LB_CUDA(up(&ctx->pring, ptabs.ring));
+    LB_CUDA(up(&ctx->prest_edge, rest_edge));
+    LB_CUDA(up(&ctx->prest_tri, rest_tri));
+    LB_CUDA(up(&ctx->prest_node, rest_node));
+    LB_CUDA(dalloc(ctx, &ctx->acc, 3 * (size_t)ctx->M));
     LB_CUDA(up(&ctx->tris, ctx->htris));
     LB_CUDA(up(&ctx->triS0, ctx->htriS0));
     LB_CUDA(up(&ctx->chunks, ctx->hchunks));
@@ -930,14 +1026,26 @@ lb_status commit_ibm(lb_ctx* ctx) {
     }
     LB_CUDA(cudaMallocHost((void**)&ctx->hq_pinned, sizeof(Q4) * (size_t)ctx->M));
     LB_CUDA(cudaMemsetAsync(ctx->F, 0, sizeof(float4) * ctx->M, ctx->stream));
-    LB_CUDA(dalloc(ctx, &ctx->partials, ctx->NCH));
+    LB_CUDA(dalloc(ctx, &ctx->partials, std::max(ctx->NCH, ctx->n_patches)));
     LB_CUDA(dalloc(ctx, &ctx->counters, ctx->C));
     LB_CUDA(cudaMemsetAsync(ctx->counters, 0, sizeof(unsigned) * ctx->C, ctx->stream));
     LB_CUDA(dalloc(ctx, &ctx->cell_sums, ctx->C));
     LB_CUDA(cudaMemsetAsync(ctx->cell_sums, 0, sizeof(double2) * ctx->C, ctx->stream));
     LB_CUDA(dalloc(ctx, &ctx->cell_rel, ctx->C));
     LB_CUDA(cudaMemsetAsync(ctx->cell_rel, 0, sizeof(float2) * ctx->C, ctx->stream));
+    LB_CUDA(cudaStreamSynchronize(ctx->stream));   // the tables above are this call's own
     return LB_OK;
+}
+
+lb_status commit_ibm(lb_ctx* ctx) {
+    if (ctx->committed) return LB_OK;
+    ctx->committed = true;
+    try {
+        return commit_tables(ctx);
+    } catch (const std::exception&) {   // (host memory; no exception leaves the library)
+        ctx->poisoned = true;
+        return fail(ctx, LB_ERR_OOM, "host memory for the membrane tables");
+    }
 }
 
 lb_status upload_channels(lb_ctx* ctx) {
@@ -1337,7 +1445,7 @@ lb_status store_step(lb_ctx* ctx, int k) {
     // programmatic dependents as in the plain cycle, except the segment's
     // first kernel (it follows the zeroing of the segment's force slots)
     ia.pdl = ctx->pdl && k > 0;
-    LB_CUDA(launch_elements(ia, s));
+    LB_CUDA(launch_membrane(ia, s));
     ia.pdl = la.pdl = ctx->pdl;
     LB_CUDA(launch_forces_spread(ia, s));
     LB_CUDA(k3_launch(ctx, la, ctx->k3, s));
@@ -1846,7 +1954,7 @@ lb_status ibm_add_mesh(lb_ctx* ctx, const double* rest_xyz, int n, const int32_t
     // the connectivity: from the context's cache when a mesh with the same
     // triangles was added before (then only the positions are checked)
     if (!rest_xyz || !tris || n < 4 || nt < 4) return fail(ctx, LB_ERR_ARG, "mesh needs >= 4 nodes and triangles");
-    const MeshConn* conn = nullptr;
+    MeshConn* conn = nullptr;
     for (const auto& c : ctx->conn_cache)
         if (c->n == n && c->nt == nt && std::memcmp(c->tris.data(), tris, sizeof(int32_t) * 3 * (size_t)nt) == 0) {
             conn = c.get();
@@ -1860,6 +1968,11 @@ lb_status ibm_add_mesh(lb_ctx* ctx, const double* rest_xyz, int n, const int32_t
         if (const char* err = build_conn(rest_xyz, n, tris, nt, *c, S0, V0)) return fail(ctx, LB_ERR_ARG, err);
         ctx->conn_cache.push_back(std::move(c));
         conn = ctx->conn_cache.back().get();
+        try {
+            const MeshConn* cc = conn;
+            conn->patches = std::async(std::launch::async, [cc] { return conn_patches(*cc); });
+        } catch (const std::exception&) {   // no thread: the commit builds them
+        }
     }
     const double* x = rest_xyz;
     const int node0 = (int)ctx->hq0.size();
@@ -1882,7 +1995,6 @@ lb_status ibm_add_mesh(lb_ctx* ctx, const double* rest_xyz, int n, const int32_t
     pm.node0 = node0;
     pm.tri0 = tri0;
     pm.e0 = ctx->n_edges_staged;
-    pm.slot0 = ctx->n_slots_staged;
     pm.cell = cell;
     pm.ch = ctx->cur;
     pm.ks = (float)mod->ks;
@@ -1890,7 +2002,6 @@ lb_status ibm_add_mesh(lb_ctx* ctx, const double* rest_xyz, int n, const int32_t
     ctx->pending_meshes.push_back(pm);
     ctx->n_tris_staged += nt;
     ctx->n_edges_staged += (int)conn->edges.size();
-    ctx->n_slots_staged += (int)conn->slots.size();
     CellDev cd;
     std::memset(&cd, 0, sizeof(cd));
     cd.ch = ctx->cur;

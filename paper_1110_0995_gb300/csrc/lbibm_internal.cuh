@@ -24,22 +24,20 @@
 //                                 groups (the stencils of the IB points)
 //   IB nodes     int64 q[2][M]x4  positions in 2^-40 lu fixed point (by parity)
 //                int64 q0[M]x4    rest positions
-//                int4 info        (cell, reference node, ring offset, valence | channel << 8)
-//   ring CSR     int4 per slot of a node's ring: where the node's share of the
-//                incident triangle, edge and opposite edge lies in the
-//                element outputs below
+//                int4 info        (cell, reference node, 0, channel << 8)
 //   edges        int4 (a, b, c, d), a < b: edge (a, b) between triangles
 //                (a, b, c) and (b, a, d); float4 (L0, theta0, ks, kb)
-//   element outputs (rewritten every step, read by the node gather):
-//                float4 eS[E]     stretching force on a (on b: its negative)
-//                float4 eB[4E]    bending force on a, b, c, d
-//                float4 tA[3T]    area direction a_k of vertex k, .w = kal dS_t/S0_t
-//                float4 tN[T]     unnormalised outward normal of the triangle
+//   patches      per distinct connectivity: the patches of at most PATCH_NODES
+//                nodes its membrane kernel works on (PatchTab), shared by all
+//                cells of that connectivity; a PatchJob per patch of a cell
+//   acc          float4[3][M] per node: local membrane force, sum of the area
+//                directions, sum of the normals (rewritten every step)
 #pragma once
 
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <utility>
+#include <vector>
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -152,6 +150,38 @@ struct CellDev {
     double S0, V0;        // rest area and volume (FP64)
 };
 
+// One patch of a mesh's nodes (indices below are local to the patch, its own
+// nodes first, then the nodes around them):
+//   loc  [n_loc]          node of the mesh
+//   tri  [n_tri]          (a | b << 16, c | owner << 31)
+//   edge [n_edge]         (a | b << 16, c | d << 16)
+//   ring [1 + rows][2 n_own]  two lanes per node, each half of its slots: row 0
+//                         the edge to the half's first neighbour; then per slot
+//                         (edge to the next neighbour | triangle << 16, opposite
+//                         edge); bit 15 of an edge to a neighbour: the node is
+//                         its b; 0xffffffff: no more slots
+struct PatchTab {
+    int n_own, n_loc, n_tri, n_edge, rows;
+    int loc0, tri0, edge0, ring0;   // offsets in the context's tables
+};
+// One block of the membrane kernel: a patch of a cell, with the cell's rest
+// data of the patch's elements and nodes in the patch's order (pq0 relative to
+// the reference node) and the cell's moduli.
+struct __align__(16) PatchJob {
+    PatchTab tab;
+    int cell, ref, node0, grid, patch0, n_patch;   // of the cell
+    int rest_edge, rest_tri, rest_node;            // offsets of its rest data
+    float ks, kb, kal;
+    int pad[3];
+};
+struct Fix3 {
+    long long x, y, z;
+};
+// Nodes per patch: 642-node red cells in 6 patches of 107, 2562-node tumor
+// cells in 24; two lanes of a 256-thread block per node.
+constexpr int PATCH_NODES = 108;
+constexpr size_t PATCH_SMEM = 40 << 10;   // shared memory of a patch; larger ones are cut further
+
 struct LatticeArgs {
     const ChannelDev* ch; // all channels (global memory)
     int n_ch;
@@ -197,25 +227,29 @@ struct IbmArgs {
     int n_ch;
     const ChannelDev* ch;
     const CellDev* cells;
-    const int4* info;     // [M] (cell, ref, ring offset, valence | channel << 8)
+    const int4* info;     // [M] (cell, ref, 0, channel << 8)
     Q4* qa;               // [M] positions, even steps
     Q4* qb;               // [M] positions, odd steps
     const Q4* q0;         // [M] rest positions
-    const int4* slots;    // [K] (3 t + role in t, 4 e + role in e, 4 e' + role in e', t) per ring slot
-    const int4* edges;    // [E] (a, b, c, d)
-    const float4* edge_rest;  // [E] (L0, theta0, ks, kb)
-    int n_edges;
-    float4* eS;           // [E]
-    float4* eB;           // [4E]
-    float4* tA;           // [3T]
-    float4* tN;           // [T]
+    // membrane kernel: one job per block, the patches' tables, the cells' rest data
+    const PatchJob* patches;
+    int n_patches, patch_smem;
+    int sm_count;
+    const uint32_t* ploc;
+    const uint2* ptri;
+    const uint2* pedge;
+    const uint2* pring;
+    const float2* prest_edge;   // (L0, theta0)
+    const float* prest_tri;     // S0_t
+    const Fix3* prest_node;     // rest position minus the reference node's
+    float4* acc;          // [3M] (F, A, N) per node
     float4* F;            // [M] last node forces
     // area / volume reduction
     const int4* tris;     // [T] (a, b, c, cell) global node indices
     const float* tri_S0;  // [T] rest area of each triangle
     const int4* chunks;   // [NCH] (cell, t_begin, t_end, chunks of that cell)
     int n_chunks;
-    longlong2* partials;  // [NCH] (dS, 6 dV) per chunk, 2^-40 units
+    longlong2* partials;  // (dS, 6 dV) per chunk or patch, 2^-40 units
     unsigned* counters;   // [C]
     double2* cell_sums;   // [C] (dS, dV)
     float2* cell_rel;     // [C] (dS / S0, dV / V0)
@@ -382,7 +416,22 @@ cudaError_t launch_diagnostics(const LatticeArgs& a, int ch_index, int n, void* 
                                const int* rep_err, const int* sched_err, double* out, cudaStream_t s);
 
 cudaError_t launch_cell_sums(const IbmArgs& a, cudaStream_t s);
-cudaError_t launch_elements(const IbmArgs& a, cudaStream_t s);
+// Connectivity of one mesh in its own numbering, and the patches built from it.
+struct MeshTables {
+    int n, nt, n_edges;
+    const int32_t* tris;
+    const int4 *edges, *slots;
+    const int *ring_off, *valence;
+};
+struct PatchTables {
+    std::vector<PatchTab> tab;
+    std::vector<uint32_t> loc;
+    std::vector<uint2> tri, edge, ring;
+    std::vector<int> tri_id, edge_id;   // triangle / edge of the mesh per entry
+};
+void build_patches(const MeshTables& m, PatchTables& out);   // host
+size_t patch_smem_bytes(const PatchTab& t);
+cudaError_t launch_membrane(const IbmArgs& a, cudaStream_t s);
 cudaError_t launch_forces_spread(const IbmArgs& a, cudaStream_t s);
 cudaError_t launch_gfix_to_g(const IbmArgs& a, cudaStream_t s);
 cudaError_t launch_interp_advance(const IbmArgs& a, cudaStream_t s);
