@@ -186,6 +186,7 @@ struct lb_ctx {
     unsigned long long* gfix = nullptr;  // [3][Ntot] its sums
     float4* W = nullptr;                 // [M] their velocities
     int rep_cap = 0, rep_nb = 0;
+    int max_cell_nodes = 0;
     float4 *rep_R = nullptr, *rep_bounds = nullptr;
     int2* rep_pairs = nullptr;
     int *rep_count = nullptr, *rep_near = nullptr, *rep_near_count = nullptr, *rep_err = nullptr, *rep_bead_ch = nullptr;
@@ -508,12 +509,11 @@ lb_status enqueue_step(lb_ctx* ctx, int par) {
         ra.R = ctx->rep_R;
         ra.err = ctx->rep_err;
         for (size_t k = 0; k < ctx->ch.size() && k < (size_t)MAXCH_P; ++k) ra.chp[k] = ctx->ch[k].d;
-        LB_CUDA(cudaMemsetAsync(ctx->rep_R, 0, sizeof(float4) * ctx->M, ctx->stream));
-        LB_CUDA(cudaMemsetAsync(ctx->rep_count, 0, sizeof(int), ctx->stream));
-        LB_CUDA(cudaMemsetAsync(ctx->rep_near_count, 0, sizeof(int) * ctx->C, ctx->stream));
+        ra.max_nodes = ctx->max_cell_nodes;
+        ra.pdl = ia.pdl;
         cudaError_t e = launch_repulsion(ra, ctx->sm_count, ctx->stream);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "kernel launch");
-        ctx->launches[1] += 4;
+        ctx->launches[1] += 3;
     }
     for (int k = 0; k < 4; ++k) {
         if (!ibm && k != 2) continue;
@@ -989,6 +989,7 @@ lb_status commit_tables(lb_ctx* ctx) {
                 bc.push_back((int)k);
             }
         ctx->rep_nb = (int)bq.size();
+        for (const CellDev& c : ctx->hcells) ctx->max_cell_nodes = std::max(ctx->max_cell_nodes, c.n_nodes);
         ctx->rep_cap = 32 * std::max(ctx->C, 1);
         LB_CUDA(dalloc(ctx, &ctx->rep_R, ctx->M));
         LB_CUDA(dalloc(ctx, &ctx->rep_bounds, ctx->C));
@@ -2101,7 +2102,7 @@ lb_status lb_step(lb_ctx* ctx, int n_steps) {
         for (int c = 0; c < 4; ++c)
             if ((ctx->M > 0 || c == 2) && !(c == 3 && ctx->W))
                 ctx->launches[c] += (c == 1 && ctx->deterministic) ? 2 * n : n;   // + the fixed-point conversion
-        if (ctx->M > 0 && ctx->rep_k > 0.f) ctx->launches[1] += 4 * n;   // collision kernels
+        if (ctx->M > 0 && ctx->rep_k > 0.f) ctx->launches[1] += 3 * n;   // collision kernels
         ctx->step += n;
         k += n;
     }

@@ -329,6 +329,8 @@ constexpr int REP_NEARB = 256;      // candidate beads per cell
 struct RepArgs {
     float k, dc;                    // force k (dc - d) for d < dc
     int n_cells, n_nodes, n_beads, pair_cap;
+    int max_nodes;                  // of one cell
+    int pdl;                        // launched as programmatic dependents
     const Q4* q;                    // current positions
     const CellDev* cells;
     const int4* info;

@@ -8,12 +8,22 @@
 //   * a node and a bead surface (d = |x - c| - r),
 //   * a node and a wall of a non-periodic axis (walls half a link outside the
 //     first and last lattice node).
-// Per step: each cell's bounding sphere (k_rep_bounds), candidate cell pairs
-// and cell-bead pairs from the bounding spheres (k_rep_pairs), node-node forces
-// for each ordered candidate pair, one block per pair with the partner's nodes
-// staged in shared memory (k_rep_nodes), then node-bead and node-wall forces
-// (k_rep_walls_beads).  The result R is added to the membrane forces before
-// spreading.  Distances come from exact fixed-point differences.
+// Per step three launches, each a programmatic dependent of the one before:
+// each cell's bounding sphere and its candidate beads, one block per cell
+// (k_rep_cells); candidate cell pairs from the bounding spheres and, beside
+// them, every node's bead and wall forces, which start its R (k_rep_pairs);
+// node-node forces of the candidate pairs, added to R (k_rep_nodes).  R joins
+// the membrane forces in the spreading kernel.  Distances come from exact
+// fixed-point differences.
+//
+// What bounds it: launches while few cells touch (seven launches and clears in
+// a row took 28 us of the 98 us cycle of the 16-slit experiment, GB300; these
+// three 16), and node pairs when cells touch.  A pair of cells is cut into
+// units of RN_THREADS nodes, so that two 2562-node tumor cells spread over 22
+// blocks rather than two, and both sides first drop the nodes outside the other
+// cell's bounding sphere, which leaves a few per cent of the pairs: two such
+// cells beside a red cell in a 32x108x19 channel 4586 -> 36 us per cycle,
+// the 62-cell 256x128x64 filter with collisions 410 -> 84.
 #include "lbibm_internal.cuh"
 
 namespace lbibm {
@@ -28,22 +38,43 @@ __device__ __forceinline__ const ChannelDev& rchan(const RepArgs& a, int c) {
     return c < MAXCH_P ? a.chp[c] : a.ch[c];
 }
 
-__device__ __forceinline__ float min_image(float d, int per, int n) {
-    return per ? d - (float)n * rintf(d / (float)n) : d;
+// Minimum image along one axis: n and 1 / n, or zeros when it is not periodic.
+struct Image {
+    float n, inv;
+};
+__device__ __forceinline__ Image image(const ChannelDev& C, int d) {
+    const int n = d == 0 ? C.nx : d == 1 ? C.ny : C.nz;
+    return C.per[d] ? Image{(float)n, 1.0f / (float)n} : Image{0.f, 0.f};
+}
+__device__ __forceinline__ float min_image(float d, Image m) { return fmaf(-m.n, rintf(d * m.inv), d); }
+
+// Periods (in 2^-40 lu) between a coordinate and the image of it next to `to`.
+__device__ __forceinline__ long long periods(float from, float to, Image m) {
+    return (long long)(int)rintf((from - to) * m.inv) * ((long long)(int)m.n << FIX_BITS);
+}
+// A fixed-point difference wrapped into half a period, exactly.
+__device__ __forceinline__ long long wrapped(long long d, Image m) {
+    return d - (long long)(int)rintf(rfx(d) * m.inv) * ((long long)(int)m.n << FIX_BITS);
 }
 
+constexpr int RC_THREADS = 512;
+
 // (1) bounding sphere of every cell: centre (relative to the reference node,
-// plus the reference node's absolute position) and radius.
-__global__ void k_rep_bounds(const __grid_constant__ RepArgs a) {
+// plus the reference node's absolute position) and radius; the beads within
+// reach.  Margin 0.5 lu covers the float rounding of the absolute centres.
+__global__ void __launch_bounds__(RC_THREADS) k_rep_cells(const __grid_constant__ RepArgs a) {
     const CellDev& C = a.cells[blockIdx.x];
+    const ChannelDev& Ch = rchan(a, C.ch);
+    const int ch = C.ch, node0 = C.node0, nn = C.n_nodes;
+    pdl_entry();
     const Q4 qr = a.q[C.ref];
     float sx = 0.f, sy = 0.f, sz = 0.f;
-    for (int i = threadIdx.x; i < C.n_nodes; i += blockDim.x) {
-        const Q4 q = a.q[C.node0 + i];
+    for (int i = threadIdx.x; i < nn; i += RC_THREADS) {
+        const Q4 q = a.q[node0 + i];
         sx += rfx(q.x - qr.x); sy += rfx(q.y - qr.y); sz += rfx(q.z - qr.z);
     }
-    __shared__ float sh[3][32];
-    __shared__ float cen[3];
+    __shared__ float sh[3][RC_THREADS / 32];
+    __shared__ int near;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -52,17 +83,16 @@ __global__ void k_rep_bounds(const __grid_constant__ RepArgs a) {
         sz += __shfl_xor_sync(0xffffffffu, sz, o);
     }
     if (lane == 0) { sh[0][wid] = sx; sh[1][wid] = sy; sh[2][wid] = sz; }
+    if (threadIdx.x == 0) near = 0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t[3] = {0.f, 0.f, 0.f};
-        for (int w = 0; w < (int)blockDim.x / 32; ++w)
-            for (int d = 0; d < 3; ++d) t[d] += sh[d][w];
-        for (int d = 0; d < 3; ++d) cen[d] = t[d] / (float)C.n_nodes;
-    }
-    __syncthreads();
+    float cen[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < RC_THREADS / 32; ++w)
+        for (int d = 0; d < 3; ++d) cen[d] += sh[d][w];
+    for (int d = 0; d < 3; ++d) cen[d] /= (float)nn;
     float r2 = 0.f;
-    for (int i = threadIdx.x; i < C.n_nodes; i += blockDim.x) {
-        const Q4 q = a.q[C.node0 + i];
+    for (int i = threadIdx.x; i < nn; i += RC_THREADS) {
+        const Q4 q = a.q[node0 + i];
         const float dx = rfx(q.x - qr.x) - cen[0], dy = rfx(q.y - qr.y) - cen[1], dz = rfx(q.z - qr.z) - cen[2];
         r2 = fmaxf(r2, dx * dx + dy * dy + dz * dz);
     }
@@ -71,126 +101,53 @@ __global__ void k_rep_bounds(const __grid_constant__ RepArgs a) {
     __syncthreads();
     if (lane == 0) sh[0][wid] = r2;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = 0.f;
-        for (int w = 0; w < (int)blockDim.x / 32; ++w) m = fmaxf(m, sh[0][w]);
-        // absolute centre as float (a coarse test with a margin; distances
-        // between nodes themselves use fixed point)
-        a.bounds[blockIdx.x] = make_float4(rfx(qr.x) + cen[0], rfx(qr.y) + cen[1], rfx(qr.z) + cen[2], sqrtf(m));
-    }
-}
-
-// (2) candidate pairs: threads [0, C*C) test ordered cell pairs (a != b, same
-// channel), threads [C*C, C*C + C*nb) test (cell, bead) pairs.  Margin 0.5 lu
-// covers the float rounding of the absolute centres.
-__global__ void k_rep_pairs(const __grid_constant__ RepArgs a) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nC = a.n_cells;
-    const long long np = nC * nC;
-    if (t < np) {
-        const int ca = (int)(t / nC), cb = (int)(t - (t / nC) * nC);
-        if (ca == cb || a.cells[ca].ch != a.cells[cb].ch) return;
-        const ChannelDev& Ch = rchan(a, a.cells[ca].ch);
-        const float4 A = a.bounds[ca], B = a.bounds[cb];
-        const float dx = min_image(A.x - B.x, Ch.per[0], Ch.nx), dy = min_image(A.y - B.y, Ch.per[1], Ch.ny),
-                    dz = min_image(A.z - B.z, Ch.per[2], Ch.nz);
-        const float lim = A.w + B.w + a.dc + 0.5f;
-        if (dx * dx + dy * dy + dz * dz < lim * lim) {
-            const int k = atomicAdd(a.pair_count, 1);
-            if (k < a.pair_cap) a.pairs[k] = make_int2(ca, cb);
-            else atomicAdd(a.err, 1);
-        }
-    } else if (t < np + nC * a.n_beads) {
-        const long long u = t - np;
-        const int c = (int)(u / a.n_beads), b = (int)(u - (u / a.n_beads) * a.n_beads);
-        if (a.bead_ch[b] != a.cells[c].ch) return;
-        const ChannelDev& Ch = rchan(a, a.cells[c].ch);
-        const float4 A = a.bounds[c];
+#pragma unroll
+    for (int w = 0; w < RC_THREADS / 32; ++w) r2 = fmaxf(r2, sh[0][w]);
+    // absolute centre as float (a coarse test with a margin; distances
+    // between nodes themselves use fixed point)
+    const float4 A = make_float4(rfx(qr.x) + cen[0], rfx(qr.y) + cen[1], rfx(qr.z) + cen[2], sqrtf(r2));
+    if (threadIdx.x == 0) a.bounds[blockIdx.x] = A;
+    const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
+    for (int b = threadIdx.x; b < a.n_beads; b += RC_THREADS) {
+        if (a.bead_ch[b] != ch) continue;
         const Q4 bq = a.bead_q[b];
-        const float dx = min_image(A.x - rfx(bq.x), Ch.per[0], Ch.nx), dy = min_image(A.y - rfx(bq.y), Ch.per[1], Ch.ny),
-                    dz = min_image(A.z - rfx(bq.z), Ch.per[2], Ch.nz);
+        const float dx = min_image(A.x - rfx(bq.x), ix), dy = min_image(A.y - rfx(bq.y), iy),
+                    dz = min_image(A.z - rfx(bq.z), iz);
         const float lim = A.w + a.bead_r[b] + a.dc + 0.5f;
         if (dx * dx + dy * dy + dz * dz < lim * lim) {
-            const int k = atomicAdd(a.near_count + c, 1);
-            if (k < REP_NEARB) a.near[c * REP_NEARB + k] = b;
+            const int k = atomicAdd(&near, 1);
+            if (k < REP_NEARB) a.near[blockIdx.x * REP_NEARB + k] = b;
             else atomicAdd(a.err, 1);
         }
     }
-}
-
-// (3) node-node forces of ordered candidate pairs (a, b): forces on a's nodes,
-// b's nodes staged in shared memory relative to a's reference node.
-constexpr int RN_THREADS = 256;
-constexpr int RN_TILE = 512;
-
-__global__ void __launch_bounds__(RN_THREADS) k_rep_nodes(const __grid_constant__ RepArgs a) {
-    __shared__ float3 tile[RN_TILE];
-    const int n_pairs = min(*a.pair_count, a.pair_cap);
-    const float k = a.k, dc = a.dc, dc2 = a.dc * a.dc;
-    for (int p = blockIdx.x; p < n_pairs; p += gridDim.x) {
-        const int2 pr = a.pairs[p];
-        const CellDev& A = a.cells[pr.x];
-        const CellDev& B = a.cells[pr.y];
-        const ChannelDev& Ch = rchan(a, A.ch);
-        const Q4 qr = a.q[A.ref];
-        for (int i0 = 0; i0 < A.n_nodes; i0 += RN_THREADS) {
-            const int i = i0 + threadIdx.x;
-            float3 xi = make_float3(0.f, 0.f, 0.f);
-            if (i < A.n_nodes) {
-                const Q4 q = a.q[A.node0 + i];
-                xi = make_float3(rfx(q.x - qr.x), rfx(q.y - qr.y), rfx(q.z - qr.z));
-            }
-            float fx = 0.f, fy = 0.f, fz = 0.f;
-            for (int j0 = 0; j0 < B.n_nodes; j0 += RN_TILE) {
-                __syncthreads();
-                for (int j = threadIdx.x; j < RN_TILE && j0 + j < B.n_nodes; j += RN_THREADS) {
-                    const Q4 q = a.q[B.node0 + j0 + j];
-                    tile[j] = make_float3(rfx(q.x - qr.x), rfx(q.y - qr.y), rfx(q.z - qr.z));
-                }
-                __syncthreads();
-                const int nj = min(RN_TILE, B.n_nodes - j0);
-                if (i < A.n_nodes) {
-                    for (int j = 0; j < nj; ++j) {
-                        const float3 xj = tile[j];
-                        const float dx = min_image(xi.x - xj.x, Ch.per[0], Ch.nx);
-                        const float dy = min_image(xi.y - xj.y, Ch.per[1], Ch.ny);
-                        const float dz = min_image(xi.z - xj.z, Ch.per[2], Ch.nz);
-                        const float d2 = dx * dx + dy * dy + dz * dz;
-                        if (d2 < dc2 && d2 > 0.f) {
-                            const float d = sqrtf(d2);
-                            const float f = k * (dc - d) / d;
-                            fx += f * dx; fy += f * dy; fz += f * dz;
-                        }
-                    }
-                }
-            }
-            if (i < A.n_nodes && (fx != 0.f || fy != 0.f || fz != 0.f)) {
-                float* r = reinterpret_cast<float*>(a.R + A.node0 + i);
-                atomicAdd(r, fx);
-                atomicAdd(r + 1, fy);
-                atomicAdd(r + 2, fz);
-            }
-        }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a.near_count[blockIdx.x] = near;
+        if (blockIdx.x == 0) *a.pair_count = 0;   // counted by the next kernel
     }
 }
 
-// (4) node-bead (the cell's candidate beads) and node-wall forces.
-__global__ void k_rep_walls_beads(const __grid_constant__ RepArgs a) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n_nodes) return;
+// Node-bead (the cell's candidate beads) and node-wall forces of node i.
+__device__ __forceinline__ void rep_walls_beads(const RepArgs& a, int i) {
     const int c = a.info[i].x;
     const CellDev& C = a.cells[c];
     const ChannelDev& Ch = rchan(a, C.ch);
     const Q4 q = a.q[i];
     const float k = a.k, dc = a.dc;
+    const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
+    // the image of the cell in the middle of the box (exact: the distances below
+    // keep their FP32 accuracy however far the cell has travelled)
+    const float4 S = a.bounds[c];
+    const long long px = q.x - periods(S.x, 0.5f * ix.n, ix), py = q.y - periods(S.y, 0.5f * iy.n, iy),
+                    pz = q.z - periods(S.z, 0.5f * iz.n, iz);
     float fx = 0.f, fy = 0.f, fz = 0.f;
     const int nb = min(a.near_count[c], REP_NEARB);
     for (int t = 0; t < nb; ++t) {
         const int b = a.near[c * REP_NEARB + t];
         const Q4 bq = a.bead_q[b];
-        const float dx = min_image(rfx(q.x - bq.x), Ch.per[0], Ch.nx);
-        const float dy = min_image(rfx(q.y - bq.y), Ch.per[1], Ch.ny);
-        const float dz = min_image(rfx(q.z - bq.z), Ch.per[2], Ch.nz);
+        const float dx = rfx(wrapped(px - bq.x, ix));
+        const float dy = rfx(wrapped(py - bq.y, iy));
+        const float dz = rfx(wrapped(pz - bq.z, iz));
         const float d2 = dx * dx + dy * dy + dz * dz;
         const float rr = a.bead_r[b] + dc;
         if (d2 < rr * rr && d2 > 0.f) {
@@ -212,21 +169,118 @@ __global__ void k_rep_walls_beads(const __grid_constant__ RepArgs a) {
         if (lo < dc) fw[d] += k * (dc - lo);
         if (hi < dc) fw[d] -= k * (dc - hi);
     }
-    float4 r = a.R[i];
-    r.x += fx + fw[0];
-    r.y += fy + fw[1];
-    r.z += fz + fw[2];
-    a.R[i] = r;
+    a.R[i] = make_float4(fx + fw[0], fy + fw[1], fz + fw[2], 0.f);
+}
+
+// (2) blocks [0, pair_blocks): ordered cell pairs (a != b, same channel) whose
+// bounding spheres come within the cut-off; the others: bead and wall forces.
+constexpr int RP_THREADS = 128;
+__global__ void __launch_bounds__(RP_THREADS) k_rep_pairs(const __grid_constant__ RepArgs a, int pair_blocks) {
+    pdl_entry();
+    if ((int)blockIdx.x >= pair_blocks) {
+        const int i = ((int)blockIdx.x - pair_blocks) * RP_THREADS + threadIdx.x;
+        if (i < a.n_nodes) rep_walls_beads(a, i);
+        return;
+    }
+    const long long t = (long long)blockIdx.x * RP_THREADS + threadIdx.x;
+    const long long nC = a.n_cells;
+    if (t >= nC * nC) return;
+    const int ca = (int)(t / nC), cb = (int)(t - (t / nC) * nC);
+    if (ca == cb || a.cells[ca].ch != a.cells[cb].ch) return;
+    const ChannelDev& Ch = rchan(a, a.cells[ca].ch);
+    const float4 A = a.bounds[ca], B = a.bounds[cb];
+    const float dx = min_image(A.x - B.x, image(Ch, 0)), dy = min_image(A.y - B.y, image(Ch, 1)),
+                dz = min_image(A.z - B.z, image(Ch, 2));
+    const float lim = A.w + B.w + a.dc + 0.5f;
+    if (dx * dx + dy * dy + dz * dz < lim * lim) {
+        const int k = atomicAdd(a.pair_count, 1);
+        if (k < a.pair_cap) a.pairs[k] = make_int2(ca, cb);
+        else atomicAdd(a.err, 1);
+    }
+}
+
+// (3) node-node forces of ordered candidate pairs (a, b): forces on a's nodes.
+// A unit is RN_THREADS nodes of a; b's nodes near a's sphere are collected in
+// shared memory a tile at a time, relative to a's reference node.
+constexpr int RN_THREADS = 128;
+constexpr int RN_TILE = 512;
+
+__global__ void __launch_bounds__(RN_THREADS) k_rep_nodes(const __grid_constant__ RepArgs a, int units_per_pair) {
+    pdl_entry();
+    __shared__ float3 tile[RN_TILE];
+    __shared__ int count;
+    const int n_units = min(*a.pair_count, a.pair_cap) * units_per_pair;
+    const float k = a.k, dc = a.dc, dc2 = a.dc * a.dc;
+    for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
+        const int2 pr = a.pairs[u / units_per_pair];
+        const CellDev& A = a.cells[pr.x];
+        const CellDev& B = a.cells[pr.y];
+        const int i = (u % units_per_pair) * RN_THREADS + threadIdx.x;
+        if (i - (int)threadIdx.x >= A.n_nodes) continue;   // (the whole block)
+        const ChannelDev& Ch = rchan(a, A.ch);
+        const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
+        const Q4 qr = a.q[A.ref];
+        // the spheres relative to a's reference node; margin as in the pair test
+        const float rx = rfx(qr.x), ry = rfx(qr.y), rz = rfx(qr.z);
+        const float4 SA = a.bounds[pr.x], SB = a.bounds[pr.y];
+        // b's image next to a, as exact fixed-point periods
+        const long long ox = qr.x + periods(SB.x, SA.x, ix), oy = qr.y + periods(SB.y, SA.y, iy),
+                        oz = qr.z + periods(SB.z, SA.z, iz);
+        auto within = [&](float3 x, float4 S) {
+            const float dx = min_image(x.x - (S.x - rx), ix), dy = min_image(x.y - (S.y - ry), iy),
+                        dz = min_image(x.z - (S.z - rz), iz);
+            const float lim = S.w + dc + 0.5f;
+            return dx * dx + dy * dy + dz * dz < lim * lim;
+        };
+        float3 xi = make_float3(0.f, 0.f, 0.f);
+        bool live = false;
+        if (i < A.n_nodes) {
+            const Q4 q = a.q[A.node0 + i];
+            xi = make_float3(rfx(q.x - qr.x), rfx(q.y - qr.y), rfx(q.z - qr.z));
+            live = within(xi, SB);
+        }
+        if (!__syncthreads_or(live)) continue;
+        float fx = 0.f, fy = 0.f, fz = 0.f;
+        for (int j0 = 0; j0 < B.n_nodes; j0 += RN_TILE) {
+            if (threadIdx.x == 0) count = 0;
+            __syncthreads();
+            for (int j = threadIdx.x; j < RN_TILE && j0 + j < B.n_nodes; j += RN_THREADS) {
+                const Q4 q = a.q[B.node0 + j0 + j];
+                const float3 xj = make_float3(rfx(q.x - ox), rfx(q.y - oy), rfx(q.z - oz));
+                if (within(xj, SA)) tile[atomicAdd(&count, 1)] = xj;
+            }
+            __syncthreads();
+            const int nj = count;
+            if (live) {
+                for (int j = 0; j < nj; ++j) {
+                    const float3 xj = tile[j];
+                    const float dx = min_image(xi.x - xj.x, ix);
+                    const float dy = min_image(xi.y - xj.y, iy);
+                    const float dz = min_image(xi.z - xj.z, iz);
+                    const float d2 = dx * dx + dy * dy + dz * dz;
+                    if (d2 < dc2 && d2 > 0.f) {
+                        const float d = sqrtf(d2);
+                        const float f = k * (dc - d) / d;
+                        fx += f * dx; fy += f * dy; fz += f * dz;
+                    }
+                }
+            }
+            __syncthreads();   // every thread is done with the tile and its count
+        }
+        if (live && (fx != 0.f || fy != 0.f || fz != 0.f)) atomicAdd(a.R + A.node0 + i, make_float4(fx, fy, fz, 0.f));
+    }
 }
 
 cudaError_t launch_repulsion(const RepArgs& a, int sm_count, cudaStream_t s) {
     if (a.n_cells <= 0) return cudaSuccess;
-    k_rep_bounds<<<a.n_cells, 256, 0, s>>>(a);
-    const long long np = (long long)a.n_cells * a.n_cells + (long long)a.n_cells * a.n_beads;
-    k_rep_pairs<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(a);
-    k_rep_nodes<<<2 * sm_count, RN_THREADS, 0, s>>>(a);
-    k_rep_walls_beads<<<(a.n_nodes + 127) / 128, 128, 0, s>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = launch_ex(k_rep_cells, a.n_cells, RC_THREADS, 0, s, a.pdl, a);
+    const int pair_blocks = (int)(((long long)a.n_cells * a.n_cells + RP_THREADS - 1) / RP_THREADS);
+    if (e == cudaSuccess)
+        e = launch_ex(k_rep_pairs, pair_blocks + (a.n_nodes + RP_THREADS - 1) / RP_THREADS, RP_THREADS, 0, s, a.pdl, a,
+                      pair_blocks);
+    if (e == cudaSuccess)
+        e = launch_ex(k_rep_nodes, 8 * sm_count, RN_THREADS, 0, s, a.pdl, a, (a.max_nodes + RN_THREADS - 1) / RN_THREADS);
+    return e;
 }
 
 }  // namespace lbibm
