@@ -10,7 +10,8 @@
 // library allocates.  Inputs and outputs are still the caller's buffers.
 //
 // The scratch array exists once per device that loads the library and stays
-// there until the process exits.  Every call shares it and it keeps the last
+// there until the process exits.  Meshes of small cells do not touch it; every
+// call with a larger one shares it and it keeps the last
 // call's contents; each call writes every partial it later reads, so nothing
 // has to start at zero.  Two calls whose kernels overlap on the GPU (different
 // streams, or different host threads) race on the array.
@@ -23,9 +24,12 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <cooperative_groups.h>
 
 #include <mutex>
 #include <vector>
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -98,6 +102,80 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Cells of up to NA_CLUSTER_TRIS triangles: one launch, a cluster of one to
+// eight blocks per cell, whose partial sums the first block reads from the
+// others' shared memory (no scratch).  What bounds the reduction is this GPU's
+// FP64 pipe (two operations per clock per SM), at few cells the latency of one
+// triangle's chain, and in two launches the gap between them.  So the volume
+// takes its cross product from the area's (a . (b - a) x (c - a) is the same
+// determinant, and cancels less), the factors 1/2 and 1/6 are applied once per
+// cell, and a cell's triangles go in equal shares of whole warps to the largest
+// cluster with which all blocks are resident at once: more blocks per cell
+// balance the SMs, fewer leave more triangles to each block's one reduction.
+// Measured on GB300, us per call, two launches -> this: one 1,280-triangle
+// cell 11.8 -> 8.2, 62 cells (87,040 triangles) 25.5 -> 16.4, 406 cells (542,720)
+// 57.3 -> 53.3 (with eight blocks for each of the 406: 72.6).  Cells beyond 32
+// chunks of 256 keep the two launches, which spread one cell over any number of SMs.
+constexpr int NA_CLUSTER = 8;
+constexpr int NA_CLUSTER_TRIS = 32 * NA_BLOCK;
+constexpr int NA_RESIDENT = 6;                // blocks per SM at 40 registers a thread
+
+// (area x 2, volume x 6) of triangle t, added to s and v.
+__device__ __forceinline__ void triangle_terms(const double* __restrict__ xyz, const int* __restrict__ tris, int t,
+                                               double& s, double& v) {
+    const int ia = tris[3 * t], ib = tris[3 * t + 1], ic = tris[3 * t + 2];
+    const double ax = xyz[3 * ia], ay = xyz[3 * ia + 1], az = xyz[3 * ia + 2];
+    const double ux = xyz[3 * ib] - ax, uy = xyz[3 * ib + 1] - ay, uz = xyz[3 * ib + 2] - az;
+    const double wx = xyz[3 * ic] - ax, wy = xyz[3 * ic + 1] - ay, wz = xyz[3 * ic + 2] - az;
+    const double nx = uy * wz - uz * wy, ny = uz * wx - ux * wz, nz = ux * wy - uy * wx;
+    s += sqrt(nx * nx + ny * ny + nz * nz);
+    v += ax * nx + ay * ny + az * nz;
+}
+
+// Block sums of s and v: s on thread 0, v on thread 16.  The first exchange
+// leaves the sums of s to a warp's lower half and those of v to its upper half,
+// which halves the FP64 additions.
+__device__ __forceinline__ double block_sums(double s, double v, double (*sh)[2]) {
+    const bool hi = threadIdx.x & 16;
+    double x = hi ? v : s;
+    const double y = __shfl_xor_sync(0xffffffffu, hi ? s : v, 16);
+    x += y;
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o, 16);
+    if ((threadIdx.x & 15) == 0) sh[threadIdx.x >> 5][hi] = x;
+    __syncthreads();
+    if (threadIdx.x == 0 || threadIdx.x == 16)
+        for (int w = 1; w < NA_BLOCK / 32; ++w) x += sh[w][hi];
+    return x;
+}
+
+__global__ void __launch_bounds__(NA_BLOCK, NA_RESIDENT)
+    k_area_volume_cluster(const double* __restrict__ xyz, const int* __restrict__ tris, const int* __restrict__ cell_start,
+                          int max_tris, double* area, double* volume) {
+    __shared__ double sh[NA_BLOCK / 32][2];
+    __shared__ double sum[2];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int c = blockIdx.y, blocks = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    // (at most max_tris, from the host's copy of the offsets: a bound for device
+    // offsets that disagree with it)
+    const int t0 = cell_start[c], n = max(0, min(cell_start[c + 1] - t0, max_tris));
+    const int share = ((n + 31) / 32 + blocks - 1) / blocks * 32;
+    const int t1 = t0 + min(n, (rank + 1) * share);
+    double s = 0.0, v = 0.0;
+    for (int t = t0 + rank * share + threadIdx.x; t < t1; t += NA_BLOCK) triangle_terms(xyz, tris, t, s, v);
+    const double x = block_sums(s, v, sh);
+    if (threadIdx.x == 0) sum[0] = x;
+    if (threadIdx.x == 16) sum[1] = x;
+    cl.sync();
+    if (rank == 0 && (threadIdx.x == 0 || threadIdx.x == 16)) {
+        const int k = threadIdx.x >> 4;
+        double S = x;
+        for (int r = 1; r < blocks; ++r) S += cl.map_shared_rank(sum, r)[k];
+        if (k == 0) area[c] = 0.5 * S;
+        else volume[c] = S / 6.0;
+    }
+    cl.sync();   // the other blocks' shared memory stays until it has been read
+}
+
 // Pass 1: block (chunk, cell) sums area and 6 x volume of up to NA_BLOCK
 // triangles of one cell in FP64 and writes one partial.
 __global__ void __launch_bounds__(NA_BLOCK) k_area_volume_partials(const double* __restrict__ xyz,
@@ -110,33 +188,12 @@ __global__ void __launch_bounds__(NA_BLOCK) k_area_volume_partials(const double*
     const int t = t0 + k * NA_BLOCK + threadIdx.x;
     if (t0 + k * NA_BLOCK >= t1) return;   // the whole block is past this cell's triangles
     double s = 0.0, v = 0.0;
-    if (t < t1) {
-        const int ia = tris[3 * t], ib = tris[3 * t + 1], ic = tris[3 * t + 2];
-        const double ax = xyz[3 * ia], ay = xyz[3 * ia + 1], az = xyz[3 * ia + 2];
-        const double bx = xyz[3 * ib], by = xyz[3 * ib + 1], bz = xyz[3 * ib + 2];
-        const double cx = xyz[3 * ic], cy = xyz[3 * ic + 1], cz = xyz[3 * ic + 2];
-        const double ux = bx - ax, uy = by - ay, uz = bz - az;
-        const double wx = cx - ax, wy = cy - ay, wz = cz - az;
-        const double nx = uy * wz - uz * wy, ny = uz * wx - ux * wz, nz = ux * wy - uy * wx;
-        s = 0.5 * sqrt(nx * nx + ny * ny + nz * nz);
-        v = ax * (by * cz - bz * cy) + ay * (bz * cx - bx * cz) + az * (bx * cy - by * cx);
-    }
-    __shared__ double sh[2][NA_BLOCK / 32];
-    s = warp_sum(s);
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = s;
-        sh[1][threadIdx.x >> 5] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S = 0.0, V = 0.0;
-        for (int w = 0; w < NA_BLOCK / 32; ++w) {
-            S += sh[0][w];
-            V += sh[1][w];
-        }
-        partials[(long long)c * max_chunks + k] = make_double2(S, V / 6.0);
-    }
+    if (t < t1) triangle_terms(xyz, tris, t, s, v);
+    __shared__ double sh[NA_BLOCK / 32][2];
+    const double x = block_sums(s, v, sh);
+    double* out = &partials[(long long)c * max_chunks + k].x;
+    if (threadIdx.x == 0) out[0] = 0.5 * x;
+    if (threadIdx.x == 16) out[1] = x / 6.0;
 }
 
 // Pass 2: one warp per cell adds the cell's partials in a fixed order.  The
@@ -184,9 +241,28 @@ extern "C" lb_status ibm_area_volume_noalloc(const double* xyz, const int32_t* t
     if (max_chunks == 0) max_chunks = 1;
     // the scratch holds one partial per (cell, chunk of 256 triangles)
     if ((long long)n_cells * max_chunks > NA_MAX_PARTIALS) return LB_ERR_ARG;
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    int max_tris = max_chunks * NA_BLOCK;
+    if (max_tris <= NA_CLUSTER_TRIS) {
+        int cluster = NA_CLUSTER;
+        while (cluster > 1 && (long long)cluster * n_cells > NA_RESIDENT * 152) cluster /= 2;
+        const double* x = xyz;
+        const int *t = tris, *c0 = cell_tri_start;
+        void* args[] = {(void*)&x, (void*)&t, (void*)&c0, (void*)&max_tris, (void*)&area, (void*)&volume};
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = cluster;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(cluster, n_cells);
+        cfg.blockDim = dim3(NA_BLOCK);
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelExC(&cfg, (const void*)k_area_volume_cluster, args) == cudaSuccess ? LB_OK : LB_ERR_CUDA;
+    }
     double2* scratch = nullptr;
     if (scratch_address(&scratch) != cudaSuccess) return LB_ERR_CUDA;
-    cudaStream_t s = (cudaStream_t)cuda_stream;
     // each launch's own status (cudaLaunchKernel returns it; an error left over
     // from an unrelated earlier call is neither consumed nor reported here)
     const double* a_xyz = xyz;
