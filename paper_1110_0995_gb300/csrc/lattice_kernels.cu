@@ -2132,7 +2132,7 @@ __device__ __forceinline__ void adj_pull(const AdjArgs& a, long long NT, int gi,
     }
 }
 
-template <bool SLOW>
+template <bool SLOW, bool FORCED>
 __device__ __forceinline__ void adj_node(const AdjArgs& a, const ChannelDev& C, int gi, int x, int y, int z) {
     const long long gp = gi;
     Nbr nb;
@@ -2143,19 +2143,14 @@ __device__ __forceinline__ void adj_node(const AdjArgs& a, const ChannelDev& C, 
 #define LBIBM_AP(I) adj_pull<I, SLOW>(a, NT, gi, nb, lk, C, y, f, lh);
     LBIBM_ALL_I(LBIBM_AP)
 #undef LBIBM_AP
-    // The pulls above read the segment store and the adjoint written two kernels
-    // back, complete when this kernel starts; only the interpolation's adjoint
-    // lam_u comes from the kernel before it.
-    pdl_entry();
     float drho, jx, jy, jz;
     moments(f, drho, jx, jy, jz);
     const float rho = 1.0f + drho;
     const float irho = 1.0f / rho;
     // IB force, the interpolation's adjoint and lam_g live on the stencil groups only
-    const bool forced = __ldg(a.fl_t + (gp >> 5)) != 0;
     float gx = C.G[0], gy = C.G[1], gz = C.G[2];
     float4 lu = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (forced) {
+    if constexpr (FORCED) {
         const float4 gs = a.g_t[gp];
         gx += gs.x; gy += gs.y; gz += gs.z;
         lu = a.lam_u[gp];
@@ -2208,7 +2203,7 @@ __device__ __forceinline__ void adj_node(const AdjArgs& a, const ChannelDev& C, 
 #pragma unroll
     for (int i = 0; i < Q; ++i)
         lo[(size_t)i * (size_t)NT + gi] = (1.0f - om) * lh[i] + lrho + ex(i) * lvx + ey(i) * lvy + ez(i) * lvz;
-    if (forced) a.lam_g[gp] = make_float4(lgx, lgy, lgz, 0.f);
+    if constexpr (FORCED) a.lam_g[gp] = make_float4(lgx, lgy, lgz, 0.f);
     if (al != 0.f) {   // phi is exactly 0 away from the beads (tanh saturates in FP32)
         const float iD2 = iD * iD;
         const float lphi = -0.5f * a.alpha * (lux * vx + luy * vy + luz * vz) * iD2 * irho -
@@ -2217,25 +2212,57 @@ __device__ __forceinline__ void adj_node(const AdjArgs& a, const ChannelDev& C, 
     }
 }
 
-__global__ void __launch_bounds__(128, 8) k_adj_collide(const __grid_constant__ AdjArgs a) {
-    // (adj_node waits for the predecessor after its pulls)
-    const ChannelDev C = a.ch;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool inr = p < C.n;
+// The step's lattice adjoint in two kernels, by 32-node group.  A group outside
+// the step's stencil set (no IB force, no interpolation) needs only the adjoint
+// of the step after it, so those groups, most of the lattice, run beside the
+// immersed-boundary chain of that later step; the stencil groups follow the
+// chain's interpolation.  (One kernel over the lattice, 28.7 us at 128x64x64, stood
+// in line with a chain of four small kernels, 24 us, which leave the chip idle:
+// 43 us per reverse cycle, now 37; GB300.  Bound by the latency of two sets of 19
+// loads per node at 64 registers; prefetching into L2 one or two waves ahead
+// changed nothing.)
+template <bool FORCED>
+__device__ __forceinline__ void adj_group(const AdjArgs& a, int grp) {
+    const ChannelDev& C = a.ch;
+    const int p = grp * GROUP + (threadIdx.x & 31);
     const long long gp = C.base + p;   // inside the channel's padded range
-    const uint8_t fslow = inr ? __ldg(a.slow + (gp >> 5)) : (uint8_t)0;
-    const bool wslow = __any_sync(0xffffffffu, fslow != 0);
-    if (!inr || solid_at(a.mask, gp)) return;   // bitmask obstacle nodes do not update
+    if (p >= C.n || solid_at(a.mask, gp)) return;   // bitmask obstacle nodes do not update
     const int r = fdiv(p, C.dnx);
     const int x = p - r * C.nx;
     const int z = fdiv(r, C.dny);
     const int y = r - z * C.ny;
-    if (wslow) adj_node<true>(a, C, (int)gp, x, y, z);
-    else adj_node<false>(a, C, (int)gp, x, y, z);
+    if (__ldg(a.slow + (gp >> 5))) adj_node<true, FORCED>(a, C, (int)gp, x, y, z);
+    else adj_node<false, FORCED>(a, C, (int)gp, x, y, z);
 }
 
+__global__ void __launch_bounds__(128, 8) k_adj_collide(const __grid_constant__ AdjArgs a) {
+    const int grp = (blockIdx.x * blockDim.x + threadIdx.x) / GROUP;
+    if (grp * GROUP >= a.ch.n || __ldg(a.fl_t + a.ch.base / GROUP + grp)) return;
+    adj_group<false>(a, grp);
+}
+
+// Each warp looks at the flags of 32 groups, a whole grid of warps apart
+// (neighbouring groups, often all in the set, go to different warps), in one load.
+__global__ void __launch_bounds__(128, 6) k_adj_collide_forced(const __grid_constant__ AdjArgs a) {
+    pdl_entry();
+    const int groups = (a.ch.n + GROUP - 1) / GROUP;
+    const int warps = gridDim.x * (blockDim.x / 32);
+    const int lane = threadIdx.x & 31;
+    const uint8_t* fl = a.fl_t + a.ch.base / GROUP;
+    for (int g0 = (blockIdx.x * blockDim.x + threadIdx.x) / 32; g0 < groups; g0 += 32 * warps) {
+        const int g = g0 + lane * warps;
+        unsigned set = __ballot_sync(0xffffffffu, g < groups && __ldg(fl + g));
+        for (; set; set &= set - 1) adj_group<true>(a, g0 + (__ffs(set) - 1) * warps);
+    }
+}
+
+const void* adj_collide_func() { return (const void*)k_adj_collide; }
+
 cudaError_t launch_adj_collide(const AdjArgs& a, cudaStream_t s) {
-    return launch_ex(k_adj_collide, (a.ch.n + 127) / 128, 128, 0, s, a.pdl, a);
+    return launch_ex(k_adj_collide, (a.ch.n + 127) / 128, 128, 0, s, false, a);
+}
+cudaError_t launch_adj_collide_forced(const AdjArgs& a, int sms, cudaStream_t s) {
+    return launch_ex(k_adj_collide_forced, min((a.ch.n + 127) / 128, 6 * sms), 128, 0, s, false, a);
 }
 
 // ---------------------------------------------------------------------------

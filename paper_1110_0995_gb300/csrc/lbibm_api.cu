@@ -635,6 +635,30 @@ bool use_overlap(const lb_ctx* ctx) {
            ctx->timing == 0 && ctx->ib_stream != nullptr;
 }
 
+// Instantiate g with every kernel but `background` at the highest priority, so
+// that the immersed-boundary chain takes SM slots as its blocks retire.
+cudaError_t instantiate_with_background(cudaGraph_t g, const void* background, cudaGraphExec_t* out) {
+    int lo = 0, hi = 0;
+    cudaDeviceGetStreamPriorityRange(&lo, &hi);
+    size_t nn = 0;
+    cudaGraphGetNodes(g, nullptr, &nn);
+    std::vector<cudaGraphNode_t> nodes(nn);
+    if (nn) cudaGraphGetNodes(g, nodes.data(), &nn);
+    for (cudaGraphNode_t nd : nodes) {
+        cudaGraphNodeType t;
+        if (cudaGraphNodeGetType(nd, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
+        cudaKernelNodeParams kp;
+        if (cudaGraphKernelNodeGetParams(nd, &kp) != cudaSuccess) continue;
+        cudaLaunchAttributeValue v;
+        std::memset(&v, 0, sizeof(v));
+        v.priority = kp.func == background ? lo : hi;
+        cudaGraphKernelNodeSetAttribute(nd, cudaLaunchAttributePriority, &v);
+    }
+    cudaGetLastError();
+    // node priorities only take effect with this flag
+    return cudaGraphInstantiateWithFlags(out, g, cudaGraphInstantiateFlagUseNodePriority);
+}
+
 lb_status build_graphs_overlap(lb_ctx* ctx) {
     for (int par = 0; par < 2; ++par)
         for (int lead = 0; lead < 2; ++lead) {
@@ -645,28 +669,8 @@ lb_status build_graphs_overlap(lb_ctx* ctx) {
             cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
             if (s != LB_OK) return s;
             if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamEndCapture");
-            // every kernel but the bulk stream-collide at the highest priority, so
-            // that the immersed-boundary chain takes SM slots as bulk blocks retire
-            int lo = 0, hi = 0;
-            cudaDeviceGetStreamPriorityRange(&lo, &hi);
-            const void* bulk = stream_collide_bulk_func((int)ctx->storage, ctx->k3.bs);
-            size_t nn = 0;
-            cudaGraphGetNodes(g, nullptr, &nn);
-            std::vector<cudaGraphNode_t> nodes(nn);
-            if (nn) cudaGraphGetNodes(g, nodes.data(), &nn);
-            for (cudaGraphNode_t nd : nodes) {
-                cudaGraphNodeType t;
-                if (cudaGraphNodeGetType(nd, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
-                cudaKernelNodeParams kp;
-                if (cudaGraphKernelNodeGetParams(nd, &kp) != cudaSuccess) continue;
-                cudaLaunchAttributeValue v;
-                std::memset(&v, 0, sizeof(v));
-                v.priority = kp.func == bulk ? lo : hi;
-                cudaGraphKernelNodeSetAttribute(nd, cudaLaunchAttributePriority, &v);
-            }
-            cudaGetLastError();
-            // node priorities only take effect with this flag
-            e = cudaGraphInstantiateWithFlags(&ctx->gexec_ov[par][lead], g, cudaGraphInstantiateFlagUseNodePriority);
+            e = instantiate_with_background(g, stream_collide_bulk_func((int)ctx->storage, ctx->k3.bs),
+                                            &ctx->gexec_ov[par][lead]);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphInstantiate");
         }
@@ -1668,7 +1672,10 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
                 cudaGraph_t g = nullptr;
                 LB_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
                 int l = lc, x = xc;
-                cudaError_t e = cudaSuccess;
+                // the lattice adjoint outside the stencil set of cycle k on the second
+                // stream, beside the immersed-boundary chain of cycle k + 1
+                cudaStream_t side = ctx->ib_stream;
+                cudaError_t e = cudaEventRecord(ctx->ev_fork[0], s);
                 for (int k = len - 1; k >= 0 && e == cudaSuccess; --k) {
                     A.q_t = W.seg_q + (size_t)k * ctx->M;
                     A.F_t = W.seg_F + (size_t)k * ctx->M;
@@ -1684,19 +1691,28 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
                     // each kernel a programmatic dependent of the one before it,
                     // except the graph's first
                     A.pdl = ctx->pdl && k < len - 1;
-                    e = launch_adj_interp(A, s);
+                    // ev_fork: the stencil groups of cycle k + 1; ev_join: the other groups of cycle k
+                    // (of k + 1, in the other slot, for the stencil groups: both read lam_in everywhere
+                    // and write the buffer that cycle k + 1 read)
+                    e = cudaStreamWaitEvent(side, ctx->ev_fork[0], 0);
+                    if (e == cudaSuccess) e = launch_adj_collide(A, side);
+                    if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_join[k & 1], side);
+                    if (e == cudaSuccess) e = launch_adj_interp(A, s);
+                    if (e == cudaSuccess && k < len - 1) e = cudaStreamWaitEvent(s, ctx->ev_join[(k + 1) & 1], 0);
+                    if (e == cudaSuccess) e = launch_adj_collide_forced(A, ctx->sm_count, s);
+                    if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_fork[0], s);
                     A.pdl = ctx->pdl;
-                    if (e == cudaSuccess) e = launch_adj_collide(A, s);
                     if (e == cudaSuccess) e = launch_adj_spread(A, s);
                     if (e == cudaSuccess) e = launch_adj_membrane(A, s);
                     l = 1 - l;
                     x = 1 - x;
                 }
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ev_join[0], 0);
                 cudaError_t e2 = cudaStreamEndCapture(s, &g);
                 if (e != cudaSuccess) return cuda_fail(ctx, e, "adjoint launch");
                 if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "cudaStreamEndCapture");
                 cudaGraphExec_t ge = nullptr;
-                e = cudaGraphInstantiate(&ge, g, 0);
+                e = instantiate_with_background(g, adj_collide_func(), &ge);
                 cudaGraphDestroy(g);
                 if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphInstantiate");
                 it = W.g_bwd.emplace(key, ge).first;

@@ -441,7 +441,9 @@ cudaError_t launch_positions_to_double(const Q4* q, int n, double* out, cudaStre
 
 cudaError_t launch_repulsion(const RepArgs& a, int sm_count, cudaStream_t s);
 cudaError_t launch_adj_interp(const AdjArgs& a, cudaStream_t s);
-cudaError_t launch_adj_collide(const AdjArgs& a, cudaStream_t s);
+cudaError_t launch_adj_collide(const AdjArgs& a, cudaStream_t s);   // groups outside the stencil set
+cudaError_t launch_adj_collide_forced(const AdjArgs& a, int sms, cudaStream_t s);   // the stencil groups
+const void* adj_collide_func();
 cudaError_t launch_adj_spread(const AdjArgs& a, cudaStream_t s);
 cudaError_t launch_adj_membrane(const AdjArgs& a, cudaStream_t s);
 cudaError_t launch_adj_bead_grad(const AdjArgs& a, cudaStream_t s);
