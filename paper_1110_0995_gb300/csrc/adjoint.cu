@@ -6,11 +6,11 @@
 //   spreading                g(x) = sum_j w(x - X_j) F_j + G
 //   membrane forces          F = F(X; ks, kb, ...)
 // each as a vector-Jacobian product written out by hand.  The adjoint of the
-// pull is a gather from the neighbours (the push, read backwards).  Element
-// Jacobians are taken in forward mode (float dual numbers), so no second
-// derivative is derived by hand: for the energy-derived edge forces one
-// evaluation along the adjoint (symmetric Jacobian), for the triangle forces
-// (the homocentric area force is not a gradient) one per input coordinate.
+// pull is a gather from the neighbours (the push, read backwards).  The edge
+// forces derive from energies (symmetric Jacobian): one forward-mode evaluation
+// (float dual numbers) along the adjoint.  The triangle forces do not (the
+// homocentric area force is not a gradient): their product with the adjoint is
+// differentiated by hand.
 // Populations are FP32 (shifted storage h = f - w; the shift is a constant).
 #include "lbibm_internal.cuh"
 
@@ -56,13 +56,7 @@ __device__ __forceinline__ V3 cross(const V3& a, const V3& b) {
     return V3{a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
 __device__ __forceinline__ V3 v3(float x, float y, float z) { return V3{mk(x), mk(y), mk(z)}; }
-__device__ __forceinline__ float tdot(const V3& a, float4 l) { return a.x.d * l.x + a.y.d * l.y + a.z.d * l.z; }
 __device__ __forceinline__ float vdot(const V3& a, float4 l) { return a.x.v * l.x + a.y.v * l.y + a.z.v * l.z; }
-__device__ __forceinline__ void seed(V3& a, int k) {
-    if (k == 0) a.x.d = 1.f;
-    else if (k == 1) a.y.d = 1.f;
-    else a.z.d = 1.f;
-}
 
 // v * 2^-40 as float (v a small fixed-point difference)
 __device__ __forceinline__ float fxa(long long v) {
@@ -124,19 +118,28 @@ __device__ __forceinline__ float sub_sum(float v, unsigned smask) {
     return v;
 }
 
-// (B1) interpolation + advance, reversed: lam_u(x_c) += w_c lamX, and
-// lamX_out = lamX + sum_c grad w_c (u(x_c) . lamX).
+// (B6, B1) lamX gets the global terms of the later cycle's membrane forces
+// (the triangle kernel left each node's sums and the cells' products): lam_S =
+// lam_c1 kag / S0 times dS/dx, lam_V = lam_c2 kv / (6 V0) times dV/dx = sum of
+// the normals / 6.  Then the interpolation and advance, reversed: lam_u(x_c) +=
+// w_c lamX, and lamX_out = lamX + sum_c grad w_c (u(x_c) . lamX).
 __global__ void k_adj_interp(const __grid_constant__ AdjArgs a) {
     pdl_entry();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    // the cycle's per-cell sums (B5) start from zero; the previous cycle's
-    // reader (B6) has completed
-    for (int k = t; k < 2 * a.n_cells; k += gridDim.x * blockDim.x) a.lam_c[k] = 0.0;
     const int j = t / ADJ_SUB, c = t & (ADJ_SUB - 1);
     if (j >= a.M) return;   // whole groups of eight lanes leave together
     const unsigned smask = 0xffu << (threadIdx.x & 24);
     const Q4 q = a.q_t[j];
-    const float4 l = a.lamX[j];
+    float4 l = a.lamX[j];
+    {
+        const int cell = a.info[j].x;
+        const float4 ds = a.sum_dS[j], n = a.sum_n[j];
+        const float lS = (float)a.lam_c[2 * cell] * a.cells[cell].kag_S0;
+        const float vn = (float)a.lam_c[2 * cell + 1] * a.cells[cell].kv_6V0 / 6.0f;
+        l.x += lS * ds.x + vn * n.x;
+        l.y += lS * ds.y + vn * n.y;
+        l.z += lS * ds.z + vn * n.z;
+    }
     float gx = 0.f, gy = 0.f, gz = 0.f;
     long long g;
     float w;
@@ -158,6 +161,9 @@ __global__ void k_adj_interp(const __grid_constant__ AdjArgs a) {
 __global__ void k_adj_spread(const __grid_constant__ AdjArgs a) {
     pdl_entry();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    // the sums of this cycle's triangles start from zero (their reader, the
+    // interpolation, has completed)
+    for (int k = t; k < 2 * a.n_cells; k += gridDim.x * blockDim.x) a.lam_c[k] = 0.0;
     const int j = t / ADJ_SUB, c = t & (ADJ_SUB - 1);
     if (j >= a.M) return;
     const unsigned smask = 0xffu << (threadIdx.x & 24);
@@ -179,6 +185,8 @@ __global__ void k_adj_spread(const __grid_constant__ AdjArgs a) {
     gx = sub_sum(gx, smask);
     gy = sub_sum(gy, smask);
     gz = sub_sum(gz, smask);
+    if (c == 1) a.sum_dS[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c == 2) a.sum_n[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c == 0) {
         a.lamF[j] = make_float4(lx, ly, lz, 0.f);
         float4 o = a.lamX_out[j];
@@ -269,61 +277,80 @@ __device__ __forceinline__ void adj_edges_block(const AdjArgs& a, int blk) {
 // ---------------------------------------------------------------------------
 // (B5) triangles: local area (with the cell's global terms held fixed),
 // global area and volume, reversed.  Force on vertex i:
-//   F_i = (kal dS_t/S0_t + c1) a_i - c2 n_t,   a_i = -(2 S_t / sum |w|^2) w_i,
-//   c1 = kag (S - S0)/S0, c2 = kv (V - V0)/(6 V0).
-// Writes the column products, accumulates per cell lam_c1 = sum lamF . a_i and
-// lam_c2 = -sum lamF . n_t, and keeps dS_t/dx_b, dS_t/dx_c and n_t for (B6).
+//   F_i = ca a_i - c2 n,   a_i = cw w_i,   w_i = x_i - mean,   n = x_b x x_c,
+//   ca = kal (S - S0)/S0 + c1,   cw = -2 S / W,   S = |n|/2,   W = sum |w_i|^2,
+//   c1 = kag (S_cell - S0_cell)/S0_cell,   c2 = kv (V - V0)/(6 V0)
+// (positions relative to vertex a).  With L = sum lamF_i and P = sum lamF_i . w_i
+// the product is ca cw P - c2 L . n, whose gradient is, by the chain rule,
+//   x_b:  x_c x N + 2 A w_b + ca cw (lamF_b - L/3)
+//   x_c:  N x x_b + 2 A w_c + ca cw (lamF_c - L/3)
+//   N = P (cw kal/S0 - 2 ca/W) n/(4 S) - c2 L,   A = 2 P ca S / W^2,
+// and minus their sum for a.  Adds the gradients, accumulates per cell lam_c1 =
+// sum lamF . a_i = cw P and lam_c2 = -L . n, and per node the sums of dS/dx and n
+// for (B6), which the next interpolation adds.
+//
+// One thread per triangle; what bounds it is the serial chain of one element
+// (gather, arithmetic, atomics), as for the edges.  Forward mode with a thread
+// per input coordinate took six threads and twelve scalar atomics per triangle
+// and a second launch for (B6): 11.1 + 3.8 us -> 6.9 us per cycle at nine
+// cells (15,360 triangles).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void tri_forces(const V3& xb, const V3& xc, float S0t, float kal, float c1, float c2,
-                                           V3 f[3], V3 av[3], V3& n, DF& St) {
-    n = cross(xb, xc);
-    St = 0.5f * dsqrt(dot(n, n));
-    const V3 third = V3{(xb.x + xc.x) / 3.0f, (xb.y + xc.y) / 3.0f, (xb.z + xc.z) / 3.0f};
-    const V3 w0 = -third, w1 = xb - third, w2 = xc - third;
-    const DF ww = dot(w0, w0) + dot(w1, w1) + dot(w2, w2);
-    const DF cw = -(2.0f * St) / ww;
-    av[0] = cw * w0; av[1] = cw * w1; av[2] = cw * w2;
-    const DF ca = kal * ((St + (-S0t)) / S0t) + c1;
-    f[0] = ca * av[0] - mk(c2) * n;
-    f[1] = ca * av[1] - mk(c2) * n;
-    f[2] = ca * av[2] - mk(c2) * n;
+__device__ __forceinline__ float3 f3(float x, float y, float z) { return make_float3(x, y, z); }
+__device__ __forceinline__ float3 cross3(float3 a, float3 b) {
+    return f3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
+__device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 
-// One thread per (triangle, column): column v*3+k seeds coordinate k of vertex
-// b or c (v = 0, 1); the column of a is minus their sum.  The column-0 thread
-// also forms the per-cell products and keeps the normal.
 __device__ __forceinline__ void adj_tris_block(const AdjArgs& a, int blk) {
-    const int tid = blk * blockDim.x + threadIdx.x;
-    const int t = tid / 6, col = tid - 6 * (tid / 6);
+    const int t = blk * blockDim.x + threadIdx.x;
     const bool valid = t < a.n_tris;   // every lane stays for the per-cell warp sums
     int cell = -1;
     float lc1 = 0.f, lc2 = 0.f;
     if (valid) {
         const int4 tr = a.tris[t];
-        const CellDev& C = a.cells[tr.w];
-        const float2 rel_sv = a.rel_t[tr.w];   // (dS/S0, dV/V0) of this step
-        const float c1 = C.kag * rel_sv.x, c2 = C.kv * rel_sv.y / 6.0f;
+        cell = tr.w;
         const Q4 qa = a.q_t[tr.x], qb = a.q_t[tr.y], qc = a.q_t[tr.z];
         const float4 la = a.lamF[tr.x], lb = a.lamF[tr.y], lc = a.lamF[tr.z];
-        V3 xb = rel(qa, qb), xc = rel(qa, qc);
-        const int v = col / 3, k = col % 3;
-        if (v == 0) seed(xb, k);
-        else seed(xc, k);
-        V3 f[3], av[3], n;
-        DF St;
-        tri_forces(xb, xc, a.tri_S0[t], C.kal, c1, c2, f, av, n, St);
-        const float acc = tdot(f[0], la) + tdot(f[1], lb) + tdot(f[2], lc);
-        atomicAdd(reinterpret_cast<float*>(a.lamX_out + (v == 0 ? tr.y : tr.z)) + k, acc);
-        atomicAdd(reinterpret_cast<float*>(a.lamX_out + tr.x) + k, -acc);
-        reinterpret_cast<float*>(a.tri_dS)[6 * t + col] = St.d;
-        if (col == 0) {
-            cell = tr.w;
-            lc1 = vdot(av[0], la) + vdot(av[1], lb) + vdot(av[2], lc);
-            lc2 = -(vdot(n, la) + vdot(n, lb) + vdot(n, lc));
-            a.tri_n[t] = make_float4(n.x.v, n.y.v, n.z.v, 0.f);
-        }
+        const CellDev& C = a.cells[cell];
+        const float2 rel_sv = a.rel_t[cell];   // (dS/S0, dV/V0) of this step
+        const float S0t = a.tri_S0[t];
+        const float c1 = C.kag * rel_sv.x, c2 = C.kv * rel_sv.y / 6.0f;
+        const float3 xb = f3(fxa(qb.x - qa.x), fxa(qb.y - qa.y), fxa(qb.z - qa.z));
+        const float3 xc = f3(fxa(qc.x - qa.x), fxa(qc.y - qa.y), fxa(qc.z - qa.z));
+        const float3 m = f3((xb.x + xc.x) / 3.0f, (xb.y + xc.y) / 3.0f, (xb.z + xc.z) / 3.0f);
+        const float3 wb = f3(xb.x - m.x, xb.y - m.y, xb.z - m.z), wc = f3(xc.x - m.x, xc.y - m.y, xc.z - m.z);
+        const float3 n = cross3(xb, xc);
+        const float S = 0.5f * sqrtf(dot3(n, n));
+        const float iW = 1.0f / (dot3(m, m) + dot3(wb, wb) + dot3(wc, wc));
+        const float cw = -2.0f * S * iW;
+        const float ca = C.kal * ((S - S0t) / S0t) + c1;
+        const float3 L = f3(la.x + lb.x + lc.x, la.y + lb.y + lc.y, la.z + lb.z + lc.z);
+        const float third = 1.0f / 3.0f;
+        const float3 eb = f3(lb.x - third * L.x, lb.y - third * L.y, lb.z - third * L.z);
+        const float3 ec = f3(lc.x - third * L.x, lc.y - third * L.y, lc.z - third * L.z);
+        const float P = dot3(eb, xb) + dot3(ec, xc);
+        const float i4S = 0.25f / S;
+        const float AS = P * (cw * C.kal / S0t - 2.0f * ca * iW) * i4S;
+        const float A2 = 4.0f * P * ca * S * iW * iW;
+        const float cc = ca * cw;
+        const float3 N = f3(AS * n.x - c2 * L.x, AS * n.y - c2 * L.y, AS * n.z - c2 * L.z);
+        const float3 gb = cross3(xc, N), gc = cross3(N, xb);
+        const float3 b = f3(gb.x + A2 * wb.x + cc * eb.x, gb.y + A2 * wb.y + cc * eb.y, gb.z + A2 * wb.z + cc * eb.z);
+        const float3 c = f3(gc.x + A2 * wc.x + cc * ec.x, gc.y + A2 * wc.y + cc * ec.y, gc.z + A2 * wc.z + cc * ec.z);
+        atomic_add3(a.lamX_out + tr.y, b.x, b.y, b.z);
+        atomic_add3(a.lamX_out + tr.z, c.x, c.y, c.z);
+        atomic_add3(a.lamX_out + tr.x, -(b.x + c.x), -(b.y + c.y), -(b.z + c.z));
+        const float3 db = cross3(xc, n), dc = cross3(n, xb);   // times 1/(4 S): dS/dx
+        atomic_add3(a.sum_dS + tr.y, i4S * db.x, i4S * db.y, i4S * db.z);
+        atomic_add3(a.sum_dS + tr.z, i4S * dc.x, i4S * dc.y, i4S * dc.z);
+        atomic_add3(a.sum_dS + tr.x, -i4S * (db.x + dc.x), -i4S * (db.y + dc.y), -i4S * (db.z + dc.z));
+        atomic_add3(a.sum_n + tr.x, n.x, n.y, n.z);
+        atomic_add3(a.sum_n + tr.y, n.x, n.y, n.z);
+        atomic_add3(a.sum_n + tr.z, n.x, n.y, n.z);
+        lc1 = cw * P;
+        lc2 = -dot3(L, n);
     }
-    // per-cell sums lam_c1, lam_c2 over the column-0 lanes: one atomic per cell per warp
+    // per-cell sums lam_c1, lam_c2: one atomic per cell per warp
     const bool has = cell >= 0;
     const int lane = threadIdx.x & 31;
     unsigned rem = __ballot_sync(AFULL, has);
@@ -346,31 +373,11 @@ __device__ __forceinline__ void adj_tris_block(const AdjArgs& a, int blk) {
 }
 
 // (B4) + (B5) in one launch: blocks [0, edge_blocks) take the edges, the rest
-// the triangle columns (the two are independent; B6 follows).
+// the triangles (the two are independent).
 __global__ void __launch_bounds__(128, 6) k_adj_membrane(const __grid_constant__ AdjArgs a, int edge_blocks) {
     pdl_entry();
     if ((int)blockIdx.x < edge_blocks) adj_edges_block(a, blockIdx.x);
     else adj_tris_block(a, (int)blockIdx.x - edge_blocks);
-}
-
-// (B6) the cell's global terms: lam_S = lam_c1 kag / S0, lam_V = lam_c2 kv / (6 V0);
-// dS/dx from the triangles' areas, dV/dx_k = sum over triangles at k of n_t / 6.
-__global__ void k_adj_tris_global(const __grid_constant__ AdjArgs a) {
-    pdl_entry();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.n_tris) return;
-    const int4 tr = a.tris[t];
-    const CellDev& C = a.cells[tr.w];
-    const float lS = (float)a.lam_c[2 * tr.w] * C.kag_S0;
-    const float lV = (float)a.lam_c[2 * tr.w + 1] * C.kv_6V0;
-    const float* ds = reinterpret_cast<const float*>(a.tri_dS) + 6 * t;
-    const float3 db = make_float3(ds[0], ds[1], ds[2]), dc = make_float3(ds[3], ds[4], ds[5]);
-    const float4 n = a.tri_n[t];
-    const float vn = lV / 6.0f;
-    atomic_add3(a.lamX_out + tr.y, lS * db.x + vn * n.x, lS * db.y + vn * n.y, lS * db.z + vn * n.z);
-    atomic_add3(a.lamX_out + tr.z, lS * dc.x + vn * n.x, lS * dc.y + vn * n.y, lS * dc.z + vn * n.z);
-    atomic_add3(a.lamX_out + tr.x, -lS * (db.x + dc.x) + vn * n.x, -lS * (db.y + dc.y) + vn * n.y,
-                -lS * (db.z + dc.z) + vn * n.z);
 }
 
 // dJ/dc_k = sum_x Lphi(x) dphi(x)/dc_k, with phi = 1 - prod_j (1 - phi_j):
@@ -437,11 +444,9 @@ cudaError_t launch_adj_spread(const AdjArgs& a, cudaStream_t s) {
     return launch_ex(k_adj_spread, (ADJ_SUB * a.M + 127) / 128, 128, 0, s, a.pdl, a);
 }
 cudaError_t launch_adj_membrane(const AdjArgs& a, cudaStream_t s) {
-    const int eb = (a.n_edges + 127) / 128, tb = (6 * a.n_tris + 127) / 128;
+    const int eb = (a.n_edges + 127) / 128, tb = (a.n_tris + 127) / 128;
     if (eb + tb == 0) return cudaSuccess;
-    cudaError_t e = launch_ex(k_adj_membrane, eb + tb, 128, 0, s, a.pdl, a, eb);
-    if (a.n_tris > 0 && e == cudaSuccess) e = launch_ex(k_adj_tris_global, (a.n_tris + 127) / 128, 128, 0, s, a.pdl, a);
-    return e;
+    return launch_ex(k_adj_membrane, eb + tb, 128, 0, s, a.pdl, a, eb);
 }
 cudaError_t launch_adj_bead_grad(const AdjArgs& a, cudaStream_t s) {
     if (a.n_beads <= 0) return cudaSuccess;

@@ -203,7 +203,7 @@ struct lb_ctx {
         float *ck_h = nullptr, *seg_h = nullptr, *fin_h = nullptr, *lam[2] = {nullptr, nullptr}, *Lphi = nullptr;
         Q4 *ck_q = nullptr, *seg_q = nullptr, *fin_q = nullptr;
         float4 *seg_F = nullptr, *seg_g = nullptr, *seg_u = nullptr, *lam_u = nullptr, *lam_g = nullptr;
-        float4 *lamX[2] = {nullptr, nullptr}, *lamF = nullptr, *tri_dS = nullptr, *tri_n = nullptr;
+        float4 *lamX[2] = {nullptr, nullptr}, *lamF = nullptr, *sum_dS = nullptr, *sum_n = nullptr;
         float4 *fin_u = nullptr, *fin_F = nullptr;
         uint8_t *seg_fl = nullptr, *fl_zero = nullptr;
         // captured segment sweeps: forward (key: len, start parity) and
@@ -1542,7 +1542,7 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
         for (void* p : {(void*)W.ck_h, (void*)W.seg_h, (void*)W.fin_h, (void*)W.lam[0], (void*)W.lam[1], (void*)W.Lphi,
                         (void*)W.ck_q, (void*)W.seg_q, (void*)W.fin_q, (void*)W.seg_F, (void*)W.seg_g, (void*)W.seg_u,
                         (void*)W.lam_u, (void*)W.lam_g, (void*)W.lamX[0], (void*)W.lamX[1], (void*)W.lamF,
-                        (void*)W.tri_dS, (void*)W.tri_n, (void*)W.seg_rel, (void*)W.lam_c, (void*)W.grad,
+                        (void*)W.sum_dS, (void*)W.sum_n, (void*)W.seg_rel, (void*)W.lam_c, (void*)W.grad,
                         (void*)W.fin_u, (void*)W.fin_F, (void*)W.seg_fl, (void*)W.fl_zero})
             dfree(ctx, p);
         for (auto& kv : W.g_fwd) cudaGraphExecDestroy(kv.second);
@@ -1573,8 +1573,8 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
         ATRY(dalloc(ctx, &W.lamX[0], ctx->M));
         ATRY(dalloc(ctx, &W.lamX[1], ctx->M));
         ATRY(dalloc(ctx, &W.lamF, ctx->M));
-        ATRY(dalloc(ctx, &W.tri_dS, 2 * (size_t)ctx->T));
-        ATRY(dalloc(ctx, &W.tri_n, ctx->T));
+        ATRY(dalloc(ctx, &W.sum_dS, ctx->M));
+        ATRY(dalloc(ctx, &W.sum_n, ctx->M));
         ATRY(dalloc(ctx, &W.lam_c, 2 * (size_t)ctx->C));
         ATRY(dalloc(ctx, &W.grad, 2 + 3 * 64));
 #undef ATRY
@@ -1616,6 +1616,9 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
     LB_CUDA(cudaMemsetAsync(W.Lphi, 0, sizeof(float) * ctx->Ntot, s));
     LB_CUDA(cudaMemsetAsync(W.lam_u, 0, sizeof(float4) * ctx->Ntot, s));
     LB_CUDA(cudaMemsetAsync(W.lam_g, 0, sizeof(float4) * ctx->Ntot, s));
+    LB_CUDA(cudaMemsetAsync(W.sum_dS, 0, sizeof(float4) * ctx->M, s));
+    LB_CUDA(cudaMemsetAsync(W.sum_n, 0, sizeof(float4) * ctx->M, s));
+    LB_CUDA(cudaMemsetAsync(W.lam_c, 0, sizeof(double) * 2 * ctx->C, s));
     LB_CUDA(cudaMemsetAsync(W.grad, 0, sizeof(double) * (2 + 3 * 64), s));
     {
         std::vector<float4> l0(ctx->M, make_float4(0.f, 0.f, 0.f, 0.f));
@@ -1650,8 +1653,8 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
     A.tri_S0 = ctx->triS0;
     A.info = ctx->info;
     A.cells = ctx->d_cells;
-    A.tri_dS = W.tri_dS;
-    A.tri_n = W.tri_n;
+    A.sum_dS = W.sum_dS;
+    A.sum_n = W.sum_n;
     A.lam_c = W.lam_c;
     A.grad = W.grad;
     int lc = 0, xc = 0;

@@ -318,8 +318,8 @@ struct AdjArgs {
     const float* tri_S0;
     const int4* info;
     const CellDev* cells;
-    float4* tri_dS;           // [2T]
-    float4* tri_n;            // [T]
+    float4* sum_dS;           // [M] sum of dS/dx over the node's triangles
+    float4* sum_n;            // [M] sum of their normals
     double* lam_c;            // [2C]
     double* grad;             // [2 + 3 n_beads] (ks, kb of the objective cell, bead centres)
 };
