@@ -627,7 +627,7 @@ __device__ __forceinline__ int sc_channel(const LatticeArgs& a, int b) {
     return lo;
 }
 
-template <class S, int NPT, int BS>
+template <class S, int NPT, int BS, int MODE = SC_ALL>
 __device__ __forceinline__ void sc_block_nodes(const LatticeArgs& a, const ChannelDev& C, int b) {
     const int lane = threadIdx.x & 31;
     const int p0 = ((b - C.blk0) * BS + (int)threadIdx.x) * NPT;   // first channel-local node of this thread
@@ -640,11 +640,11 @@ __device__ __forceinline__ void sc_block_nodes(const LatticeArgs& a, const Chann
             // the block is a piece of one row: y and z are the block's
             const int r = fdiv(pb, C.dnx);
             const int z = fdiv(r, C.dny);
-            sc_nodes<S, 1, SC_ALL, true>(a, C, p0, lane, pb - r * C.nx + (int)threadIdx.x, r - z * C.ny, z);
+            sc_nodes<S, 1, MODE, true>(a, C, p0, lane, pb - r * C.nx + (int)threadIdx.x, r - z * C.ny, z);
             return;
         }
     }
-    sc_nodes<S, NPT, SC_ALL>(a, C, p0, lane);
+    sc_nodes<S, NPT, MODE>(a, C, p0, lane);
 }
 
 // ONE: a single channel, whose constants stay in the parameter bank (which is
@@ -1678,14 +1678,13 @@ __global__ void __launch_bounds__(BS, 512 / BS) k_stream_collide_pipe(const __gr
     }
 }
 
-// Differentiable variant (one node per thread).
+// Differentiable variant (one node per thread; a context of one channel, its
+// constants in the parameter bank).  As the plain kernel it loads FP32
+// populations before it waits for the spreading; waiting at the kernel's start
+// cost 0.9 of 26.3 us per cycle (128x64x64, nine cells, GB300).
 template <class S, int BS>
 __global__ void __launch_bounds__(BS, K3MinBlocks<S, 1, BS>::value) k_stream_collide_brinkman(const __grid_constant__ LatticeArgs a) {
-    pdl_entry();
-    const int b = sc_block(a);
-    const int c = sc_channel(a, b);
-    const ChannelDev C = chan(a, c);
-    sc_nodes<S, 1, SC_BRINK>(a, C, (b - C.blk0) * BS + (int)threadIdx.x, threadIdx.x & 31);
+    sc_block_nodes<S, 1, BS, SC_BRINK>(a, a.chp[0], sc_block(a));
 }
 
 // Solid fraction of the differentiable variant at every node of a channel:
