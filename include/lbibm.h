@@ -353,12 +353,13 @@ lb_status ibm_get_area_volume(lb_ctx* ctx, double* area, double* volume);
  * asynchronous.  Scratch is a fixed 1 MiB device array (65,536 partial sums
  * of 256 triangles each) that every GPU loading the library holds until the
  * process exits: LB_ERR_ARG when n_cells times the largest number of
- * 256-triangle chunks of one cell exceeds 65,536, or n_cells > 65,535.  The
+ * 256-triangle chunks of one cell exceeds 65,536, or n_cells > 65,535
+ * (meshes whose cells all have at most 8,192 triangles leave it untouched).  The
  * first call on a device looks the array's address up (cudaGetSymbolAddress)
  * and so does the first call after the device's current context changed (a
  * cudaDeviceReset, or another driver context made current); make such a call
- * before any stream capture.  Every call shares the array, so calls that
- * overlap on the GPU race.  LB_ERR_CUDA when a launch is refused; an error
+ * before any stream capture.  Every other call shares the array, so such
+ * calls that overlap on the GPU race.  LB_ERR_CUDA when a launch is refused; an error
  * left over from an earlier, unrelated call is not consumed.  Calls no
  * cudaMalloc or cudaFree.  n_cells = 0 does nothing and returns LB_OK. */
 lb_status ibm_area_volume_noalloc(const double* xyz, const int32_t* tris, const int32_t* cell_tri_start,
@@ -420,9 +421,9 @@ lb_status lb_get_step(lb_ctx* ctx, int64_t* step);
 lb_status lb_save_state(lb_ctx* ctx, void* buf, size_t* bytes);
 lb_status lb_load_state(lb_ctx* ctx, const void* buf, size_t bytes);
 
-/* Optional per-kernel timing.  Kernel classes: 0 = element pass (cell area /
- * volume sums and element forces),
- * 1 = membrane forces + spreading, 2 = fused stream-collide,
+/* Optional per-kernel timing.  Kernel classes: 0 = membrane kernel (cell area /
+ * volume sums and local membrane forces per node),
+ * 1 = node forces + spreading, 2 = fused stream-collide,
  * 3 = interpolation + advance.  With kernel_mask != 0 (bit k for class k,
  * 15 = all) lb_step launches the kernels one by one (no graph) and records a
  * pair of CUDA events on the context's stream around every launch of a

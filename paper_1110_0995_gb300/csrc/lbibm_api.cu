@@ -24,8 +24,7 @@ using namespace lbibm;
 
 namespace {
 
-constexpr int CHUNK_TRIS = 128;     // triangles per block of the area/volume reduction (one per thread;
-                                    // measured on GB300: 256 -> 128 took the element pass 18.2 -> 16.5 us, 64 slower)
+constexpr int CHUNK_TRIS = 128;     // triangles per block of the area/volume reduction (one per thread)
 constexpr int MAX_VALENCE = 64;
 
 struct ChannelHost {
@@ -575,7 +574,7 @@ lb_status build_graphs(lb_ctx* ctx) {
 // One cycle in the overlapped schedule.  Only the 32-node groups of the
 // stencil set D (the groups any IB point can reach within one step, computed
 // during the previous step) depend on this step's IB forces, so
-//   ib stream:   [interpolation + advance of the previous step], elements,
+//   ib stream:   [interpolation + advance of the previous step], membrane,
 //                forces + spreading (which also marks the next step's D),
 //                compaction of the next D into a list
 //   main stream: stream-collide of every group outside D
@@ -826,7 +825,7 @@ void apply_k3_config(lb_ctx* ctx, K3Config c) {
     ctx->total_blocks = blk;
 }
 
-// The element and ring tables of every mesh (triangles with their rest
+// The element tables of every mesh (triangles with their rest
 // areas, edges with rest length and rest dihedral angle (the bending's
 // theta0, Sec. 2.3.1)), written at the commit, the
 // meshes spread over up to 16 host threads (each writes only its own ranges).
@@ -2008,7 +2007,7 @@ lb_status ibm_add_mesh(lb_ctx* ctx, const double* rest_xyz, int n, const int32_t
         ctx->hq.push_back(q);
     }
     ctx->hrest.insert(ctx->hrest.end(), x, x + 3 * (size_t)n);
-    // the element and ring tables are written when the context commits
+    // the element tables are written when the context commits
     // (every mesh's ranges at once, on host threads)
     PendingMesh pm;
     pm.conn = conn;

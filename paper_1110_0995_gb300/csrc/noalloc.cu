@@ -11,9 +11,9 @@
 //
 // The scratch array exists once per device that loads the library and stays
 // there until the process exits.  Meshes of small cells do not touch it; every
-// call with a larger one shares it and it keeps the last
-// call's contents; each call writes every partial it later reads, so nothing
-// has to start at zero.  Two calls whose kernels overlap on the GPU (different
+// call with a larger cell shares it, and it keeps the last such call's
+// contents; each call writes every partial it later reads, so nothing has to
+// start at zero.  Two such calls whose kernels overlap on the GPU (different
 // streams, or different host threads) race on the array.
 //
 // The array's device address belongs to the CUDA context that loaded the
@@ -242,6 +242,9 @@ extern "C" lb_status ibm_area_volume_noalloc(const double* xyz, const int32_t* t
     // the scratch holds one partial per (cell, chunk of 256 triangles)
     if ((long long)n_cells * max_chunks > NA_MAX_PARTIALS) return LB_ERR_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
+    // looked up on either path: any call before a capture prepares every later one
+    double2* scratch = nullptr;
+    if (scratch_address(&scratch) != cudaSuccess) return LB_ERR_CUDA;
     int max_tris = max_chunks * NA_BLOCK;
     if (max_tris <= NA_CLUSTER_TRIS) {
         int cluster = NA_CLUSTER;
@@ -261,8 +264,6 @@ extern "C" lb_status ibm_area_volume_noalloc(const double* xyz, const int32_t* t
         cfg.numAttrs = 1;
         return cudaLaunchKernelExC(&cfg, (const void*)k_area_volume_cluster, args) == cudaSuccess ? LB_OK : LB_ERR_CUDA;
     }
-    double2* scratch = nullptr;
-    if (scratch_address(&scratch) != cudaSuccess) return LB_ERR_CUDA;
     // each launch's own status (cudaLaunchKernel returns it; an error left over
     // from an unrelated earlier call is neither consumed nor reported here)
     const double* a_xyz = xyz;
