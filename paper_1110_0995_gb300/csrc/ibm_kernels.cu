@@ -339,19 +339,38 @@ __global__ void __launch_bounds__(FS_BLOCK, MASSIVE ? IB_MIN_BLOCKS : LBIBM_FS_M
     int4 inf = make_int4(0, 0, 0, 0);
     Q4 qi = {};
     long long g = 0;
-    float w = 0.f;
+    float w = 0.f, kag = 0.f, kv = 0.f;
     bool hit = false;
+    float3 U = make_float3(0.f, 0.f, 0.f);
+    float4 W = make_float4(0.f, 0.f, 0.f, 0.f);
     if (live) {
         inf = a.info[i];
+        kag = a.cells[inf.x].kag;
+        kv = a.cells[inf.x].kv;
         qi = (a.par ? a.qb : a.qa)[i];
+        if (MASSIVE) W = a.W[i];
         hit = corner(chan(a, inf.w >> 8), qi, sl, g, w);
         if (hit) hit = !((__ldg(a.mask + (g >> 5)) >> (g & 31)) & 1u);
+        if (MASSIVE) {
+            // also the point's velocity and the fluid velocity of the last
+            // collision at X (this lane's corner, summed over the eight lanes),
+            // both written two or more kernels back (loaded after the wait they
+            // cost a one-cell channel 0.6 us per cycle, GB300)
+            float4 uc = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (hit) uc = a.u[g];
+            U = make_float3(w * uc.x, w * uc.y, w * uc.z);
+            const unsigned smask = 0xffu << (threadIdx.x & 24);
+#pragma unroll
+            for (int o = SUB / 2; o > 0; o >>= 1) {
+                U.x += __shfl_xor_sync(smask, U.x, o);
+                U.y += __shfl_xor_sync(smask, U.y, o);
+                U.z += __shfl_xor_sync(smask, U.z, o);
+            }
+        }
     }
     pdl_entry();
     if (!live) return;   // whole groups of eight lanes leave together
-    const unsigned smask = 0xffu << (threadIdx.x & 24);
     const int cid = inf.x, chn = inf.w >> 8;
-    const CellDev& C = a.cells[cid];
     const ChannelDev Ch = chan(a, chn);
     if (a.dcur) {
         // overlapped schedule: the target must be in this step's stencil set
@@ -361,27 +380,16 @@ __global__ void __launch_bounds__(FS_BLOCK, MASSIVE ? IB_MIN_BLOCKS : LBIBM_FS_M
         mark_box(Ch, qi, sl, a.dmark);
     }
 
-    const float3 F = node_force(a, i, C.kag, C.kv, cid);
+    const float3 F = node_force(a, i, kag, kv, cid);
     if (sl == 0) a.F[i] = make_float4(F.x, F.y, F.z, 0.f);
 
     uint8_t* fl = a.par ? a.fl1 : a.fl0;
     const unsigned active = __activemask();
     float3 S = F;   // what reaches the fluid
     if (MASSIVE) {
-        // points with mass (Sec. 2.2 Newton equation): the fluid velocity of
-        // the last collision at X (this lane's corner, summed over the eight
-        // lanes), kick by F, exact drag drift; the fluid receives the drag's
-        // impulse and the point moves now (no interpolation kernel follows)
-        float4 uc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (hit) uc = a.u[g];
-        float3 U = make_float3(w * uc.x, w * uc.y, w * uc.z);
-#pragma unroll
-        for (int o = SUB / 2; o > 0; o >>= 1) {
-            U.x += __shfl_xor_sync(smask, U.x, o);
-            U.y += __shfl_xor_sync(smask, U.y, o);
-            U.z += __shfl_xor_sync(smask, U.z, o);
-        }
-        const float4 W = a.W[i];
+        // points with mass (Sec. 2.2 Newton equation): kick by F, exact drag
+        // drift around U; the fluid receives the drag's impulse and the point
+        // moves now (no interpolation kernel follows)
         const float3 D = make_float3(W.x + F.x * a.ib_inv_m - U.x, W.y + F.y * a.ib_inv_m - U.y,
                                      W.z + F.z * a.ib_inv_m - U.z);   // V - U
         S = make_float3(a.ib_gp1 * D.x, a.ib_gp1 * D.y, a.ib_gp1 * D.z);
