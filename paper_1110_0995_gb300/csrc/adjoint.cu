@@ -244,6 +244,7 @@ __device__ __forceinline__ void adj_edges_block(const AdjArgs& a, int blk) {
     if (e < a.n_edges) {
         const int4 ev = a.edges[e];
         const float4 er = a.edge_rest[e];   // (L0, theta0, ks, kb)
+        const int obj = __ldg(a.obj_cell);
         const Q4 qa = a.q_t[ev.x], qb = a.q_t[ev.y], qc = a.q_t[ev.z], qd = a.q_t[ev.w];
         const float4 la = a.lamF[ev.x], lb = a.lamF[ev.y], lc = a.lamF[ev.z], ld = a.lamF[ev.w];
         V3 xb = rel(qa, qb), xc = rel(qa, qc), xd = rel(qa, qd);
@@ -256,7 +257,7 @@ __device__ __forceinline__ void adj_edges_block(const AdjArgs& a, int blk) {
         atomic_add3(a.lamX_out + ev.y, fs[1].x.d + fb[1].x.d, fs[1].y.d + fb[1].y.d, fs[1].z.d + fb[1].z.d);
         atomic_add3(a.lamX_out + ev.z, fb[2].x.d, fb[2].y.d, fb[2].z.d);
         atomic_add3(a.lamX_out + ev.w, fb[3].x.d, fb[3].y.d, fb[3].z.d);
-        if (a.info[ev.x].x == a.obj_cell) {
+        if (a.info[ev.x].x == obj) {
             // parameter gradients (the forces are linear in ks and kb)
             if (er.z != 0.f) gks = (vdot(fs[0], la) + vdot(fs[1], lb)) / er.z;
             if (er.w != 0.f) gkb = (vdot(fb[0], la) + vdot(fb[1], lb) + vdot(fb[2], lc) + vdot(fb[3], ld)) / er.w;

@@ -210,6 +210,7 @@ struct lb_ctx {
         std::map<std::pair<int, int>, cudaGraphExec_t> g_fwd, g_bwd;
         float2* seg_rel = nullptr;
         double *lam_c = nullptr, *grad = nullptr;
+        int* obj = nullptr;            // the objective's cell, read by the reverse sweeps
     } adj;
     int bulk_res = 10;             // resident bulk blocks per SM (128 threads)
     int pf_nodes = 0;              // stream-collide L2 prefetch distance (lattice nodes, 0: PREFETCH_BYTES)
@@ -705,6 +706,11 @@ void drop_graphs(lb_ctx* ctx) {
                 cudaGraphExecDestroy(ctx->gexec_ov[par][lead]);
                 ctx->gexec_ov[par][lead] = nullptr;
             }
+    }
+    // the adjoint's sweeps hold the same kernel arguments (alpha, the variant)
+    for (auto* graphs : {&ctx->adj.g_fwd, &ctx->adj.g_bwd}) {
+        for (auto& kv : *graphs) cudaGraphExecDestroy(kv.second);
+        graphs->clear();
     }
 }
 
@@ -1290,8 +1296,6 @@ lb_status lb_destroy(lb_ctx* ctx) {
     if (!ctx) return LB_OK;
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_graphs(ctx);
-    for (auto& kv : ctx->adj.g_fwd) cudaGraphExecDestroy(kv.second);
-    for (auto& kv : ctx->adj.g_bwd) cudaGraphExecDestroy(kv.second);
     for (void* p : ctx->allocations) cudaFree(p);
     if (ctx->hq_pinned) cudaFreeHost(ctx->hq_pinned);
     if (ctx->diag_out) cudaFreeHost(ctx->diag_out);
@@ -1541,7 +1545,7 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
         for (void* p : {(void*)W.ck_h, (void*)W.seg_h, (void*)W.fin_h, (void*)W.lam[0], (void*)W.lam[1], (void*)W.Lphi,
                         (void*)W.ck_q, (void*)W.seg_q, (void*)W.fin_q, (void*)W.seg_F, (void*)W.seg_g, (void*)W.seg_u,
                         (void*)W.lam_u, (void*)W.lam_g, (void*)W.lamX[0], (void*)W.lamX[1], (void*)W.lamF,
-                        (void*)W.sum_dS, (void*)W.sum_n, (void*)W.seg_rel, (void*)W.lam_c, (void*)W.grad,
+                        (void*)W.sum_dS, (void*)W.sum_n, (void*)W.seg_rel, (void*)W.lam_c, (void*)W.grad, (void*)W.obj,
                         (void*)W.fin_u, (void*)W.fin_F, (void*)W.seg_fl, (void*)W.fl_zero})
             dfree(ctx, p);
         for (auto& kv : W.g_fwd) cudaGraphExecDestroy(kv.second);
@@ -1576,6 +1580,7 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
         ATRY(dalloc(ctx, &W.sum_n, ctx->M));
         ATRY(dalloc(ctx, &W.lam_c, 2 * (size_t)ctx->C));
         ATRY(dalloc(ctx, &W.grad, 2 + 3 * 64));
+        ATRY(dalloc(ctx, &W.obj, 1));
 #undef ATRY
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -1623,6 +1628,7 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
         std::vector<float4> l0(ctx->M, make_float4(0.f, 0.f, 0.f, 0.f));
         for (int i = 0; i < mo->n; ++i) l0[mo->node0 + i].x = (float)(1.0 / mo->n);   // dJ / dX^T
         LB_CUDA(cudaMemcpyAsync(W.lamX[0], l0.data(), sizeof(float4) * ctx->M, cudaMemcpyHostToDevice, s));
+        LB_CUDA(cudaMemcpyAsync(W.obj, &mo->cell, sizeof(int), cudaMemcpyHostToDevice, s));
         LB_CUDA(cudaStreamSynchronize(s));
     }
     AdjArgs A;
@@ -1632,7 +1638,7 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
     A.n_edges = ctx->E;
     A.n_tris = ctx->T;
     A.n_beads = nb;
-    A.obj_cell = mo->cell;
+    A.obj_cell = W.obj;
     A.n_cells = ctx->C;
     A.plane = ctx->plane;
     A.mask = ctx->mask;

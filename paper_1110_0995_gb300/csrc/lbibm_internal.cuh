@@ -283,7 +283,8 @@ struct IbmArgs {
 // differentiable variant; single channel, FP32 populations).
 struct AdjArgs {
     ChannelDev ch;
-    int M, n_edges, n_tris, n_beads, obj_cell;
+    int M, n_edges, n_tris, n_beads;
+    const int* obj_cell;      // cell of the objective (device: the captured sweeps serve every objective)
     int n_cells;
     int pdl;                  // launched as a programmatic dependent of the previous kernel
     long long plane;          // population plane stride
