@@ -1591,6 +1591,7 @@ lb_status lb_adjoint(lb_ctx* ctx, int n_steps, int ckpt_every, int objective_mes
     }
     cudaStream_t s = ctx->stream;
     const long long step0 = ctx->step;
+    LB_CUDA(cudaStreamSynchronize(s));   // earlier steps may still be moving the points (mean_x copies on no stream of theirs)
     const double x0 = mean_x(ctx->q[ctx->step & 1], *mo);
     const size_t hb = sizeof(float) * hN;
     // forward: checkpoints at the start of every segment; the last segment

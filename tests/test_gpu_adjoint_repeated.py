@@ -1,5 +1,5 @@
 """lb_adjoint several times on one context: another objective mesh or another
-Brinkman coefficient.
+Brinkman coefficient; and right after steps that still run on the device.
 The reference is the same call with another checkpoint interval, which is the
 same gradient from newly captured sweeps (the workspace is of another shape)."""
 import numpy as np
@@ -59,3 +59,16 @@ def test_another_alpha():
         sim.set_brinkman(bead, alpha=0.5)
     got, want = a.adjoint(T, ckpt_every=T, objective_mesh=0), b.adjoint(T, ckpt_every=T // 2, objective_mesh=0)
     _same(got, want)
+
+
+def test_objective_right_after_steps():
+    (a, _), (b, _) = _sim(), _sim()
+    for sim in (a, b):
+        sim.adjoint(T, ckpt_every=T, objective_mesh=0)      # (the workspace is there: no call below waits for an allocation)
+        sim.step(400)
+    b.synchronize()
+    x = b.nodes(0)[:, 0].mean()
+    got = a.adjoint(T, ckpt_every=T, objective_mesh=0)
+    want = b.adjoint(T, ckpt_every=T, objective_mesh=0)
+    assert got["J"] == pytest.approx(want["J"], rel=1e-4)
+    assert want["J"] == pytest.approx(b.nodes(0)[:, 0].mean() - x, rel=1e-4)
