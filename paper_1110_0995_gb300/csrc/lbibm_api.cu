@@ -283,8 +283,8 @@ cudaError_t dalloc(lb_ctx* ctx, T** p, size_t count) {
     const size_t gz = ctx->guard;
     cudaError_t e = cudaMalloc(&v, bytes + 2 * gz);
     if (e == cudaSuccess && gz) {
-        e = cudaMemset(v, GUARD_PATTERN, gz);
-        if (e == cudaSuccess) e = cudaMemset((char*)v + gz + bytes, GUARD_PATTERN, gz);
+        e = cudaMemsetAsync(v, GUARD_PATTERN, gz, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync((char*)v + gz + bytes, GUARD_PATTERN, gz, ctx->stream);
         if (e != cudaSuccess) {
             cudaFree(v);
             v = nullptr;
@@ -1093,11 +1093,11 @@ lb_status lb_check_guard_zones(lb_ctx* ctx, int self_test, int64_t* damaged_byte
     if (ctx->guarded.empty()) return LB_OK;
     unsigned long long* d_count = nullptr;
     LB_CUDA(cudaMalloc(&d_count, sizeof(unsigned long long)));   // outside the guarded set
-    cudaError_t e = cudaMemset(d_count, 0, sizeof(unsigned long long));
+    cudaError_t e = cudaMemsetAsync(d_count, 0, sizeof(unsigned long long), ctx->stream);
     // self test: one byte of every zone changed from the host first, then restored
     for (const auto& g : ctx->guarded) {
-        if (e == cudaSuccess && self_test) e = cudaMemset(g.base + g.guard - 1, 0, 1);
-        if (e == cudaSuccess && self_test) e = cudaMemset(g.base + g.guard + g.bytes, 0, 1);
+        if (e == cudaSuccess && self_test) e = cudaMemsetAsync(g.base + g.guard - 1, 0, 1, ctx->stream);
+        if (e == cudaSuccess && self_test) e = cudaMemsetAsync(g.base + g.guard + g.bytes, 0, 1, ctx->stream);
         if (e == cudaSuccess) k_guard_count<<<8, 256, 0, ctx->stream>>>((const unsigned char*)g.base, g.guard, d_count);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e == cudaSuccess)
@@ -1109,10 +1109,11 @@ lb_status lb_check_guard_zones(lb_ctx* ctx, int self_test, int64_t* damaged_byte
     if (e == cudaSuccess) e = cudaMemcpy(&h, d_count, sizeof(h), cudaMemcpyDeviceToHost);
     if (self_test) {
         for (const auto& g : ctx->guarded) {
-            if (e == cudaSuccess) e = cudaMemset(g.base + g.guard - 1, GUARD_PATTERN, 1);
-            if (e == cudaSuccess) e = cudaMemset(g.base + g.guard + g.bytes, GUARD_PATTERN, 1);
+            if (e == cudaSuccess) e = cudaMemsetAsync(g.base + g.guard - 1, GUARD_PATTERN, 1, ctx->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(g.base + g.guard + g.bytes, GUARD_PATTERN, 1, ctx->stream);
         }
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     cudaFree(d_count);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lb_check_guard_zones");
     *damaged_bytes = (int64_t)h;
@@ -2382,14 +2383,16 @@ lb_status lb_set_populations(lb_ctx* ctx, const double* f) {
                     hs[(size_t)i * n + p] = (float)v;
                 }
             }
+    // copies on the context's stream, where the next step finds them complete
     const int par = (int)(ctx->step & 1);
     const size_t eb = pop_bytes(ctx->storage);
+    std::vector<uint16_t> h16(ctx->storage == LB_F32 ? 0 : (size_t)Q * n);
     for (int i = 0; i < Q; ++i) {
         char* dst = (char*)ctx->h[par] + ((size_t)i * ctx->plane + d.base) * eb;
         if (ctx->storage == LB_F32) {
-            LB_CUDA(cudaMemcpy(dst, hs.data() + (size_t)i * n, sizeof(float) * n, cudaMemcpyHostToDevice));
+            LB_CUDA(cudaMemcpyAsync(dst, hs.data() + (size_t)i * n, sizeof(float) * n, cudaMemcpyHostToDevice, ctx->stream));
         } else {
-            std::vector<uint16_t> tmp(n);
+            uint16_t* tmp = h16.data() + (size_t)i * n;
             for (long long p = 0; p < n; ++p) {
                 const float s = hs[(size_t)i * n + p] * (1.0f / wgt(i));
                 if (ctx->storage == LB_F16_SHIFTED) {
@@ -2400,9 +2403,10 @@ lb_status lb_set_populations(lb_ctx* ctx, const double* f) {
                     std::memcpy(&tmp[p], &bv, 2);
                 }
             }
-            LB_CUDA(cudaMemcpy(dst, tmp.data(), 2 * n, cudaMemcpyHostToDevice));
+            LB_CUDA(cudaMemcpyAsync(dst, tmp, 2 * n, cudaMemcpyHostToDevice, ctx->stream));
         }
     }
+    LB_CUDA(cudaStreamSynchronize(ctx->stream));
     return LB_OK;
 }
 
@@ -2622,18 +2626,24 @@ lb_status lb_load_state(lb_ctx* ctx, const void* buf, size_t bytes) {
     const char* p = (const char*)buf + sizeof(hd);
     ctx->step = hd.step;
     const int par = (int)(ctx->step & 1);
-    LB_CUDA(cudaStreamSynchronize(ctx->stream));
-    LB_CUDA(cudaMemcpy(ctx->h[par], p, hb, cudaMemcpyHostToDevice)); p += hb;
-    LB_CUDA(cudaMemcpy(ctx->g[1 - par], p, gb, cudaMemcpyHostToDevice)); p += gb;
-    LB_CUDA(cudaMemcpy(ctx->fl[1 - par], p, fb, cudaMemcpyHostToDevice)); p += fb;
-    LB_CUDA(cudaMemset(ctx->g[par], 0, gb));
-    LB_CUDA(cudaMemset(ctx->fl[par], 0, fb));
+    // on the context's stream: the default stream's copies and clears may end
+    // after the call that issued them, and the next step does not wait for them
+    auto load = [&](void* dst, size_t n) {
+        const cudaError_t e = cudaMemcpyAsync(dst, p, n, cudaMemcpyHostToDevice, ctx->stream);
+        p += n;
+        return e;
+    };
+    LB_CUDA(load(ctx->h[par], hb));
+    LB_CUDA(load(ctx->g[1 - par], gb));
+    LB_CUDA(load(ctx->fl[1 - par], fb));
+    LB_CUDA(cudaMemsetAsync(ctx->g[par], 0, gb, ctx->stream));
+    LB_CUDA(cudaMemsetAsync(ctx->fl[par], 0, fb, ctx->stream));
     if (ctx->M) {
-        LB_CUDA(cudaMemcpy(ctx->q[par], p, qb, cudaMemcpyHostToDevice)); p += qb;
-        LB_CUDA(cudaMemcpy(ctx->F, p, Fb, cudaMemcpyHostToDevice)); p += Fb;
+        LB_CUDA(load(ctx->q[par], qb));
+        LB_CUDA(load(ctx->F, Fb));
         if (ctx->W) {
-            LB_CUDA(cudaMemcpy(ctx->W, p, Wb, cudaMemcpyHostToDevice)); p += Wb;
-            LB_CUDA(cudaMemcpy(ctx->u, p, ub, cudaMemcpyHostToDevice)); p += ub;
+            LB_CUDA(load(ctx->W, Wb));
+            LB_CUDA(load(ctx->u, ub));
         }
         ctx->dvalid = false;
     }
