@@ -28,7 +28,11 @@
 
 namespace lbibm {
 
-__device__ __forceinline__ float rfx(long long v) {   // v * 2^-40 (|v| < 2^51)
+// v * 2^-40.  Below 2048 lu: the integer's upper and lower parts in FP32, one
+// rounding of their sum; beyond (absolute coordinates): the 64-bit integer
+// rounded to 24 bits, on the FP64 pipe.
+__device__ __forceinline__ float rfx(long long v) {
+    if (v >= (1LL << 51) || v < -(1LL << 51)) return __ll2float_rn(v) * FIX_INV_F;
     const int hi = (int)(v >> 20);
     const int lo = (int)(v & 0xFFFFF);
     return fmaf((float)hi, 9.5367431640625e-07f, (float)lo * FIX_INV_F);
@@ -48,6 +52,15 @@ __device__ __forceinline__ Image image(const ChannelDev& C, int d) {
 }
 __device__ __forceinline__ float min_image(float d, Image m) { return fmaf(-m.n, rintf(d * m.inv), d); }
 
+// Periods (in 2^-40 lu) between an absolute coordinate and its image next to
+// the origin.  Positions are never wrapped; every absolute coordinate is taken
+// minus these periods of its cell's reference node (exact), so that it is
+// about a box at most and its FP32 rounding does not grow with the distance
+// travelled.
+__device__ __forceinline__ long long home(long long q, Image m) {
+    return (long long)(int)rintf(rfx(q) * m.inv) * ((long long)(int)m.n << FIX_BITS);
+}
+
 // Periods (in 2^-40 lu) between a coordinate and the image of it next to `to`.
 __device__ __forceinline__ long long periods(float from, float to, Image m) {
     return (long long)(int)rintf((from - to) * m.inv) * ((long long)(int)m.n << FIX_BITS);
@@ -60,8 +73,9 @@ __device__ __forceinline__ long long wrapped(long long d, Image m) {
 constexpr int RC_THREADS = 512;
 
 // (1) bounding sphere of every cell: centre (relative to the reference node,
-// plus the reference node's absolute position) and radius; the beads within
-// reach.  Margin 0.5 lu covers the float rounding of the absolute centres.
+// plus the reference node's position less its periods) and radius; the beads
+// within reach.  Margin 0.5 lu covers the float rounding of the centres (on an
+// axis without periods up to 2^20 lu from the origin).
 __global__ void __launch_bounds__(RC_THREADS) k_rep_cells(const __grid_constant__ RepArgs a) {
     const CellDev& C = a.cells[blockIdx.x];
     const ChannelDev& Ch = rchan(a, C.ch);
@@ -103,16 +117,18 @@ __global__ void __launch_bounds__(RC_THREADS) k_rep_cells(const __grid_constant_
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < RC_THREADS / 32; ++w) r2 = fmaxf(r2, sh[0][w]);
-    // absolute centre as float (a coarse test with a margin; distances
-    // between nodes themselves use fixed point)
-    const float4 A = make_float4(rfx(qr.x) + cen[0], rfx(qr.y) + cen[1], rfx(qr.z) + cen[2], sqrtf(r2));
-    if (threadIdx.x == 0) a.bounds[blockIdx.x] = A;
+    // centre as float (a coarse test with a margin; distances between nodes
+    // themselves use fixed point)
     const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
+    const float4 A = make_float4(rfx(qr.x - home(qr.x, ix)) + cen[0], rfx(qr.y - home(qr.y, iy)) + cen[1],
+                                 rfx(qr.z - home(qr.z, iz)) + cen[2], sqrtf(r2));
+    if (threadIdx.x == 0) a.bounds[blockIdx.x] = A;
     for (int b = threadIdx.x; b < a.n_beads; b += RC_THREADS) {
         if (a.bead_ch[b] != ch) continue;
         const Q4 bq = a.bead_q[b];
-        const float dx = min_image(A.x - rfx(bq.x), ix), dy = min_image(A.y - rfx(bq.y), iy),
-                    dz = min_image(A.z - rfx(bq.z), iz);
+        const float dx = min_image(A.x - rfx(bq.x - home(bq.x, ix)), ix),
+                    dy = min_image(A.y - rfx(bq.y - home(bq.y, iy)), iy),
+                    dz = min_image(A.z - rfx(bq.z - home(bq.z, iz)), iz);
         const float lim = A.w + a.bead_r[b] + a.dc + 0.5f;
         if (dx * dx + dy * dy + dz * dz < lim * lim) {
             const int k = atomicAdd(&near, 1);
@@ -138,8 +154,10 @@ __device__ __forceinline__ void rep_walls_beads(const RepArgs& a, int i) {
     // the image of the cell in the middle of the box (exact: the distances below
     // keep their FP32 accuracy however far the cell has travelled)
     const float4 S = a.bounds[c];
-    const long long px = q.x - periods(S.x, 0.5f * ix.n, ix), py = q.y - periods(S.y, 0.5f * iy.n, iy),
-                    pz = q.z - periods(S.z, 0.5f * iz.n, iz);
+    const Q4 qr = a.q[C.ref];
+    const long long px = q.x - home(qr.x, ix) - periods(S.x, 0.5f * ix.n, ix),
+                    py = q.y - home(qr.y, iy) - periods(S.y, 0.5f * iy.n, iy),
+                    pz = q.z - home(qr.z, iz) - periods(S.z, 0.5f * iz.n, iz);
     float fx = 0.f, fy = 0.f, fz = 0.f;
     const int nb = min(a.near_count[c], REP_NEARB);
     for (int t = 0; t < nb; ++t) {
@@ -219,13 +237,15 @@ __global__ void __launch_bounds__(RN_THREADS) k_rep_nodes(const __grid_constant_
         if (i - (int)threadIdx.x >= A.n_nodes) continue;   // (the whole block)
         const ChannelDev& Ch = rchan(a, A.ch);
         const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
-        const Q4 qr = a.q[A.ref];
-        // the spheres relative to a's reference node; margin as in the pair test
-        const float rx = rfx(qr.x), ry = rfx(qr.y), rz = rfx(qr.z);
+        const Q4 qr = a.q[A.ref], qb = a.q[B.ref];
+        // the spheres relative to a's reference node (less its periods); margin as in the pair test
+        const long long hx = qr.x - home(qr.x, ix), hy = qr.y - home(qr.y, iy), hz = qr.z - home(qr.z, iz);
+        const float rx = rfx(hx), ry = rfx(hy), rz = rfx(hz);
         const float4 SA = a.bounds[pr.x], SB = a.bounds[pr.y];
         // b's image next to a, as exact fixed-point periods
-        const long long ox = qr.x + periods(SB.x, SA.x, ix), oy = qr.y + periods(SB.y, SA.y, iy),
-                        oz = qr.z + periods(SB.z, SA.z, iz);
+        const long long ox = hx + home(qb.x, ix) + periods(SB.x, SA.x, ix),
+                        oy = hy + home(qb.y, iy) + periods(SB.y, SA.y, iy),
+                        oz = hz + home(qb.z, iz) + periods(SB.z, SA.z, iz);
         auto within = [&](float3 x, float4 S) {
             const float dx = min_image(x.x - (S.x - rx), ix), dy = min_image(x.y - (S.y - ry), iy),
                         dz = min_image(x.z - (S.z - rz), iz);
