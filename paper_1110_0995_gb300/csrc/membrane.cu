@@ -80,6 +80,27 @@ __device__ __forceinline__ void split(long long v, int sh, float grid, float& hi
     lo = (float)(int)(v - ((long long)n << sh)) * FIX_INV_F;
 }
 
+// Node k where hi would be rounded (beyond 2^24 grid steps) or the remainder
+// is no 32-bit integer (a grid coarser than 2^-8): hi is the value itself
+// rounded to 24 bits, lo what that leaves, by 64-bit conversions.  Where the
+// kernel has 80 registers the node takes this in place of the ordinary form;
+// at 64 a second look at the patch's nodes, when any needs it, keeps the
+// ordinary loop as it was (512x256x128, membrane kernel: in place 3.7 % slower,
+// second look 1.5 % faster; 256x128x64 with the second look 13 % slower, in
+// place no different).
+__device__ __forceinline__ void far_node(const Nodes& S, int k, const Q4& q, const Q4& qr, const Fix3& x0) {
+    auto put = [](long long v, float& hi, float& lo) {
+        hi = __ll2float_rn(v) * FIX_INV_F;
+        lo = __ll2float_rn(v - __float2ll_rn(hi * FIX_SCALE_F)) * FIX_INV_F;
+    };
+    put(q.x - qr.x, S.A[k].x, S.A[k].w);
+    put(q.y - qr.y, S.A[k].y, S.B[k].x);
+    put(q.z - qr.z, S.A[k].z, S.B[k].y);
+    put(q.x - qr.x - x0.x, S.B[k].z, S.C[k].y);
+    put(q.y - qr.y - x0.y, S.B[k].w, S.C[k].z);
+    put(q.z - qr.z - x0.z, S.C[k].x, S.C[k].w);
+}
+
 __device__ __forceinline__ long long to_fixed_f(float u) {   // round(u 2^40), |u| < 2^15
     const float s = u * 65536.0f;
     const float m = rintf(s);
@@ -209,6 +230,9 @@ __global__ void __launch_bounds__(MB, MINB) k_membrane(const __grid_constant__ I
     if (!a.W) pdl_entry();
     const Q4* qc = a.par ? a.qb : a.qa;
     const Q4 qr = qc[J.ref];
+    // half of 2^24 grid steps; none for a grid coarser than 2^-8
+    const unsigned far_limit = J.grid >= 8 ? 1u << (31 - J.grid) : 0u;
+    bool far = false;
     for (int k = tid; k < tp.n_loc; k += MB) {
         if (k != tid) {
             id = (int)loc[k];
@@ -216,6 +240,11 @@ __global__ void __launch_bounds__(MB, MINB) k_membrane(const __grid_constant__ I
         }
         const Q4 q = qc[J.node0 + id];
         const long long x = q.x - qr.x, y = q.y - qr.y, z = q.z - qr.z;
+        // (the upper halves' magnitudes, 2^-8 lu; displacements are within the rest extent of the positions)
+        auto is_far = [&] {
+            auto mag = [](long long v) { return (unsigned)((int)(v >> 32) ^ (int)(v >> 63)); };
+            return (mag(x) | mag(y) | mag(z)) >= far_limit;
+        };
         float4 A, B, Cc;
         auto fill = [&](int sh, float grid) {
             split(x, sh, grid, A.x, A.w);
@@ -225,13 +254,25 @@ __global__ void __launch_bounds__(MB, MINB) k_membrane(const __grid_constant__ I
             split(y - x0.y, sh, grid, B.w, Cc.z);
             split(z - x0.z, sh, grid, Cc.x, Cc.w);
         };
+        if constexpr (MINB == 3) {
+            if (is_far()) {
+                far_node(S, k, q, qr, x0);
+                continue;
+            }
+        }
         if (J.grid == 16) fill(FIX_BITS - 16, 1.0f / 65536.0f);
         else fill(FIX_BITS - J.grid, __int_as_float((127 - J.grid) << 23));
+        if constexpr (MINB != 3) far = far || is_far();
         S.A[k] = A;
         S.B[k] = B;
         S.C[k] = Cc;
     }
-    __syncthreads();
+    if constexpr (MINB == 3) {
+        __syncthreads();
+    } else if (__syncthreads_or(far)) {
+        for (int k = tid; k < tp.n_loc; k += MB) far_node(S, k, qc[J.node0 + (int)loc[k]], qr, rest_node[k]);
+        __syncthreads();
+    }
     // elements
     long long s = 0, v = 0;
 #pragma unroll
