@@ -187,6 +187,7 @@ struct lb_ctx {
     int rep_cap = 0, rep_nb = 0;
     int max_cell_nodes = 0;
     float4 *rep_R = nullptr, *rep_bounds = nullptr;
+    int4* rep_home = nullptr;
     int2* rep_pairs = nullptr;
     int *rep_count = nullptr, *rep_near = nullptr, *rep_near_count = nullptr, *rep_err = nullptr, *rep_bead_ch = nullptr;
     Q4* rep_bead_q = nullptr;
@@ -499,6 +500,7 @@ lb_status enqueue_step(lb_ctx* ctx, int par) {
         ra.info = ctx->info;
         ra.ch = ctx->d_ch;
         ra.bounds = ctx->rep_bounds;
+        ra.home = ctx->rep_home;
         ra.pairs = ctx->rep_pairs;
         ra.pair_count = ctx->rep_count;
         ra.near = ctx->rep_near;
@@ -988,12 +990,16 @@ lb_status commit_tables(lb_ctx* ctx) {
         std::vector<int> bc;
         for (size_t k = 0; k < ctx->ch.size(); ++k)
             for (size_t b = 0; b + 3 < ctx->ch[k].spheres.size(); b += 4) {
-                Q4 q;
-                q.x = to_fixed(ctx->ch[k].spheres[b]);
-                q.y = to_fixed(ctx->ch[k].spheres[b + 1]);
-                q.z = to_fixed(ctx->ch[k].spheres[b + 2]);
-                q.w = 0;
-                bq.push_back(q);
+                // the centre's image inside the box on periodic axes
+                const ChannelDev& d = ctx->ch[k].d;
+                const int n[3] = {d.nx, d.ny, d.nz};
+                long long c[3];
+                for (int a = 0; a < 3; ++a) {
+                    double x = ctx->ch[k].spheres[b + a];
+                    if (d.per[a]) x -= n[a] * std::floor(x / n[a]);
+                    c[a] = to_fixed(x);
+                }
+                bq.push_back(Q4{c[0], c[1], c[2], 0});
                 br.push_back(ctx->ch[k].spheres[b + 3]);
                 bc.push_back((int)k);
             }
@@ -1002,6 +1008,7 @@ lb_status commit_tables(lb_ctx* ctx) {
         ctx->rep_cap = 32 * std::max(ctx->C, 1);
         LB_CUDA(dalloc(ctx, &ctx->rep_R, ctx->M));
         LB_CUDA(dalloc(ctx, &ctx->rep_bounds, ctx->C));
+        LB_CUDA(dalloc(ctx, &ctx->rep_home, ctx->C));
         LB_CUDA(dalloc(ctx, &ctx->rep_pairs, ctx->rep_cap));
         LB_CUDA(dalloc(ctx, &ctx->rep_count, 1));
         LB_CUDA(dalloc(ctx, &ctx->rep_near, (size_t)ctx->C * REP_NEARB));

@@ -336,12 +336,13 @@ struct RepArgs {
     const CellDev* cells;
     const int4* info;
     const ChannelDev* ch;
-    float4* bounds;                 // [C] centre (absolute), radius
+    int4* home;                     // [C] periods between the reference node and its image next to the origin
+    float4* bounds;                 // [C] centre (less those periods), radius
     int2* pairs;                    // [pair_cap] ordered candidate cell pairs
     int* pair_count;
     int* near;                      // [C][REP_NEARB] candidate beads per cell
     int* near_count;                // [C]
-    const Q4* bead_q;               // [nb] bead centres in fixed point
+    const Q4* bead_q;               // [nb] bead centres in fixed point, inside the box on periodic axes
     const float* bead_r;            // [nb]
     const int* bead_ch;             // [nb]
     float4* R;                      // [M] collision force per node (accumulated)

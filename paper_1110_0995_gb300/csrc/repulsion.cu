@@ -28,14 +28,13 @@
 
 namespace lbibm {
 
-// v * 2^-40.  Below 2048 lu: the integer's upper and lower parts in FP32, one
-// rounding of their sum; beyond (absolute coordinates): the 64-bit integer
-// rounded to 24 bits, on the FP64 pipe.
+// v * 2^-40: the nearest multiple of 2^32 and the rest, each rounded to FP32,
+// and their sum (below 2^-9 lu one rounding, beyond at most three quarters of
+// an ulp), over the whole range and with no 64-bit conversion.
 __device__ __forceinline__ float rfx(long long v) {
-    if (v >= (1LL << 51) || v < -(1LL << 51)) return __ll2float_rn(v) * FIX_INV_F;
-    const int hi = (int)(v >> 20);
-    const int lo = (int)(v & 0xFFFFF);
-    return fmaf((float)hi, 9.5367431640625e-07f, (float)lo * FIX_INV_F);
+    const int lo = (int)v;
+    const int hi = (int)((v + 0x80000000LL) >> 32);
+    return fmaf((float)hi, 0.00390625f, (float)lo * FIX_INV_F);   // 2^-8
 }
 
 __device__ __forceinline__ const ChannelDev& rchan(const RepArgs& a, int c) {
@@ -52,22 +51,20 @@ __device__ __forceinline__ Image image(const ChannelDev& C, int d) {
 }
 __device__ __forceinline__ float min_image(float d, Image m) { return fmaf(-m.n, rintf(d * m.inv), d); }
 
-// Periods (in 2^-40 lu) between an absolute coordinate and its image next to
-// the origin.  Positions are never wrapped; every absolute coordinate is taken
-// minus these periods of its cell's reference node (exact), so that it is
-// about a box at most and its FP32 rounding does not grow with the distance
-// travelled.
-__device__ __forceinline__ long long home(long long q, Image m) {
-    return (long long)(int)rintf(rfx(q) * m.inv) * ((long long)(int)m.n << FIX_BITS);
+// Positions are never wrapped; every absolute coordinate of a cell is taken
+// less the whole periods of its reference node (RepArgs::home, exact), so that
+// it is about a box at most and its FP32 rounding does not grow with the
+// distance travelled.
+__device__ __forceinline__ int home(long long q, Image m) { return (int)rintf(rfx(q) * m.inv); }
+__device__ __forceinline__ long long shift(int periods, Image m) {
+    return (long long)periods * ((long long)(int)m.n << FIX_BITS);
 }
 
-// Periods (in 2^-40 lu) between a coordinate and the image of it next to `to`.
-__device__ __forceinline__ long long periods(float from, float to, Image m) {
-    return (long long)(int)rintf((from - to) * m.inv) * ((long long)(int)m.n << FIX_BITS);
-}
+// Periods between a coordinate and the image of it next to `to`.
+__device__ __forceinline__ int periods(float from, float to, Image m) { return (int)rintf((from - to) * m.inv); }
 // A fixed-point difference wrapped into half a period, exactly.
 __device__ __forceinline__ long long wrapped(long long d, Image m) {
-    return d - (long long)(int)rintf(rfx(d) * m.inv) * ((long long)(int)m.n << FIX_BITS);
+    return d - shift(home(d, m), m);
 }
 
 constexpr int RC_THREADS = 512;
@@ -120,15 +117,18 @@ __global__ void __launch_bounds__(RC_THREADS) k_rep_cells(const __grid_constant_
     // centre as float (a coarse test with a margin; distances between nodes
     // themselves use fixed point)
     const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
-    const float4 A = make_float4(rfx(qr.x - home(qr.x, ix)) + cen[0], rfx(qr.y - home(qr.y, iy)) + cen[1],
-                                 rfx(qr.z - home(qr.z, iz)) + cen[2], sqrtf(r2));
-    if (threadIdx.x == 0) a.bounds[blockIdx.x] = A;
+    const int hx = home(qr.x, ix), hy = home(qr.y, iy), hz = home(qr.z, iz);
+    const float4 A = make_float4(rfx(qr.x - shift(hx, ix)) + cen[0], rfx(qr.y - shift(hy, iy)) + cen[1],
+                                 rfx(qr.z - shift(hz, iz)) + cen[2], sqrtf(r2));
+    if (threadIdx.x == 0) {
+        a.bounds[blockIdx.x] = A;
+        a.home[blockIdx.x] = make_int4(hx, hy, hz, 0);
+    }
     for (int b = threadIdx.x; b < a.n_beads; b += RC_THREADS) {
         if (a.bead_ch[b] != ch) continue;
         const Q4 bq = a.bead_q[b];
-        const float dx = min_image(A.x - rfx(bq.x - home(bq.x, ix)), ix),
-                    dy = min_image(A.y - rfx(bq.y - home(bq.y, iy)), iy),
-                    dz = min_image(A.z - rfx(bq.z - home(bq.z, iz)), iz);
+        const float dx = min_image(A.x - rfx(bq.x), ix), dy = min_image(A.y - rfx(bq.y), iy),
+                    dz = min_image(A.z - rfx(bq.z), iz);
         const float lim = A.w + a.bead_r[b] + a.dc + 0.5f;
         if (dx * dx + dy * dy + dz * dz < lim * lim) {
             const int k = atomicAdd(&near, 1);
@@ -154,10 +154,10 @@ __device__ __forceinline__ void rep_walls_beads(const RepArgs& a, int i) {
     // the image of the cell in the middle of the box (exact: the distances below
     // keep their FP32 accuracy however far the cell has travelled)
     const float4 S = a.bounds[c];
-    const Q4 qr = a.q[C.ref];
-    const long long px = q.x - home(qr.x, ix) - periods(S.x, 0.5f * ix.n, ix),
-                    py = q.y - home(qr.y, iy) - periods(S.y, 0.5f * iy.n, iy),
-                    pz = q.z - home(qr.z, iz) - periods(S.z, 0.5f * iz.n, iz);
+    const int4 H = a.home[c];
+    const long long px = q.x - shift(H.x + periods(S.x, 0.5f * ix.n, ix), ix),
+                    py = q.y - shift(H.y + periods(S.y, 0.5f * iy.n, iy), iy),
+                    pz = q.z - shift(H.z + periods(S.z, 0.5f * iz.n, iz), iz);
     float fx = 0.f, fy = 0.f, fz = 0.f;
     const int nb = min(a.near_count[c], REP_NEARB);
     for (int t = 0; t < nb; ++t) {
@@ -237,15 +237,16 @@ __global__ void __launch_bounds__(RN_THREADS) k_rep_nodes(const __grid_constant_
         if (i - (int)threadIdx.x >= A.n_nodes) continue;   // (the whole block)
         const ChannelDev& Ch = rchan(a, A.ch);
         const Image ix = image(Ch, 0), iy = image(Ch, 1), iz = image(Ch, 2);
-        const Q4 qr = a.q[A.ref], qb = a.q[B.ref];
+        const Q4 qr = a.q[A.ref];
         // the spheres relative to a's reference node (less its periods); margin as in the pair test
-        const long long hx = qr.x - home(qr.x, ix), hy = qr.y - home(qr.y, iy), hz = qr.z - home(qr.z, iz);
-        const float rx = rfx(hx), ry = rfx(hy), rz = rfx(hz);
         const float4 SA = a.bounds[pr.x], SB = a.bounds[pr.y];
+        const int4 HA = a.home[pr.x], HB = a.home[pr.y];
+        const long long hx = qr.x - shift(HA.x, ix), hy = qr.y - shift(HA.y, iy), hz = qr.z - shift(HA.z, iz);
+        const float rx = rfx(hx), ry = rfx(hy), rz = rfx(hz);
         // b's image next to a, as exact fixed-point periods
-        const long long ox = hx + home(qb.x, ix) + periods(SB.x, SA.x, ix),
-                        oy = hy + home(qb.y, iy) + periods(SB.y, SA.y, iy),
-                        oz = hz + home(qb.z, iz) + periods(SB.z, SA.z, iz);
+        const long long ox = hx + shift(HB.x + periods(SB.x, SA.x, ix), ix),
+                        oy = hy + shift(HB.y + periods(SB.y, SA.y, iy), iy),
+                        oz = hz + shift(HB.z + periods(SB.z, SA.z, iz), iz);
         auto within = [&](float3 x, float4 S) {
             const float dx = min_image(x.x - (S.x - rx), ix), dy = min_image(x.y - (S.y - ry), iy),
                         dz = min_image(x.z - (S.z - rz), iz);
