@@ -247,11 +247,12 @@ lb_status lb_get_kernel_config(lb_ctx* ctx, int* nodes_per_thread, int* block_si
  * populations (every direction's plane) of the nodes nodes_ahead past its
  * own, so that blocks running later find their pulls in L2 rather than in
  * HBM.  A performance setting only (Sec. 2.1's update is unchanged; results
- * are bit-identical for every distance).  0 (the default): the library's own
- * distance, five megabytes of populations (65,536 nodes in FP32, 131,072 in
- * 16 bits); otherwise a multiple of 256 up to 2^24, else LB_ERR_ARG.  The
- * bound on the useful distance is the L2 (19 x 4 bytes per node of distance
- * for FP32 storage). */
+ * are bit-identical for every distance).  0 = off; otherwise a multiple of
+ * 256 up to 2^24, else LB_ERR_ARG.  The bound on the useful distance is the L2
+ * (19 x 4 bytes per node of distance for FP32 storage).  A context for which
+ * none was set uses the library's own distance, five megabytes of populations
+ * (65,536 nodes in FP32, 131,072 in 16 bits; off on lattices with fewer).
+ * lb_get_prefetch: the distance in use. */
 lb_status lb_set_prefetch(lb_ctx* ctx, int nodes_ahead);
 lb_status lb_get_prefetch(lb_ctx* ctx, int* nodes_ahead);
 
@@ -279,8 +280,8 @@ lb_status lb_get_schedule(lb_ctx* ctx, int* overlapped);
 
 /* Autotuner: times every supported stream-collide variant on this context's
  * lattice (`repeats` launches each, CUDA events), selects the fastest, then
- * times its L2 prefetch distances (0, 65536, 131072, 262144 nodes; variants
- * with 1, 2 or 4 nodes per thread) and keeps the fastest (lb_get_prefetch
+ * times its L2 prefetch distances (off, 65536, 131072, 262144 nodes, as far as
+ * the lattice reaches; variants with 1, 2 or 4 nodes per thread) and keeps the fastest (lb_get_prefetch
  * reads it), and returns the variant with its mean time per launch in ms.
  * Only before the first lb_step (LB_ERR_STATE otherwise): there, repeated
  * launches leave the state unchanged. */

@@ -214,7 +214,7 @@ struct lb_ctx {
         int* obj = nullptr;            // the objective's cell, read by the reverse sweeps
     } adj;
     int bulk_res = 10;             // resident bulk blocks per SM (128 threads)
-    int pf_nodes = 0;              // stream-collide L2 prefetch distance (lattice nodes, 0: PREFETCH_BYTES)
+    int pf_nodes = -1;             // stream-collide L2 prefetch distance (lattice nodes; 0: off, -1: not set, prefetch_nodes)
     long long smem_per_sm = 0;
     // timing
     int timing = 0;          // bit k: record events around kernel class k (no graph)
@@ -323,12 +323,19 @@ __global__ void k_guard_count(const unsigned char* __restrict__ p, size_t n, uns
 
 size_t pop_bytes(lb_storage s) { return s == LB_F32 ? 4 : 2; }
 
-// The stream-collide's own L2 prefetch distance (lb_set_prefetch 0): five
+// The stream-collide's L2 prefetch distance where none was set: five
 // megabytes of populations, 65,536 nodes in FP32 and 131,072 in 16 bits, about
 // what the resident blocks hold in flight (GB300, without / with: 256x128x64
 // FP32 60.0 / 57.2 us, 512x256x128 FP32 411 / 409, FP16 261 / 246; half the
 // distance 1-4 us slower, twice no faster).
 constexpr int PREFETCH_BYTES = Q * 65536 * 4;
+// The distance in use: the set one, or the library's own, 0 where the lattice
+// has no node that far ahead.
+int prefetch_nodes(const lb_ctx* ctx) {
+    if (ctx->pf_nodes >= 0) return ctx->pf_nodes;
+    const int d = PREFETCH_BYTES / (Q * (int)pop_bytes(ctx->storage));
+    return d < ctx->Ntot ? d : 0;
+}
 // Odd steps walk the blocks backwards when both population buffers together
 // are about the size of L2 (126 MB, three quarters to three halves): they then
 // begin with what the previous step wrote last.  Measured on GB300: 181x75x53
@@ -364,7 +371,7 @@ LatticeArgs lattice_args(const lb_ctx* ctx, int par) {
     a.dlist = ctx->dlist[par];
     a.dcount = ctx->dcount ? ctx->dcount + par : nullptr;
     a.tma_err = ctx->sched_err ? ctx->sched_err + 1 : nullptr;
-    a.pf_nodes = ctx->pf_nodes > 0 ? ctx->pf_nodes : PREFETCH_BYTES / (Q * (int)pop_bytes(ctx->storage));
+    a.pf_nodes = prefetch_nodes(ctx);
     if (a.pf_nodes >= ctx->Ntot) a.pf_nodes = 0;   // nothing that far ahead
     const size_t pops = 2 * (size_t)Q * ctx->plane * pop_bytes(ctx->storage);
     a.rev = par && !ctx->phi && pops >= ZIGZAG_MIN && pops <= ZIGZAG_MAX;
@@ -2167,7 +2174,7 @@ lb_status lb_set_prefetch(lb_ctx* ctx, int nodes_ahead) {
 
 lb_status lb_get_prefetch(lb_ctx* ctx, int* nodes_ahead) {
     LB_GUARD(ctx);
-    if (nodes_ahead) *nodes_ahead = ctx->pf_nodes;
+    if (nodes_ahead) *nodes_ahead = prefetch_nodes(ctx);
     return LB_OK;
 }
 
@@ -2232,15 +2239,17 @@ lb_status lb_autotune(lb_ctx* ctx, int repeats, int* nodes_per_thread, int* bloc
         }
     }
     // then the L2 prefetch distance of the winner (variants with 1, 2 or 4
-    // nodes per thread); the distance kept is the fastest, 0 on a tie
+    // nodes per thread): off and the distances that the lattice reaches; the
+    // one kept is the fastest, the shorter on a tie
     apply_k3_config(ctx, best);
     if (ctx->ch.size() > (size_t)MAXCH_P && upload_channels(ctx) != LB_OK) return LB_ERR_CUDA;
     const int keep_pf = ctx->pf_nodes;
-    int best_pf = 0;
+    int best_pf = keep_pf;
     if (best.npt > 0) {
         const int dists[] = {0, 65536, 131072, 262144};
         double best_pf_ms = 1e30;
         for (int d : dists) {
+            if (d >= ctx->Ntot) continue;
             ctx->pf_nodes = d;
             const LatticeArgs la = lattice_args(ctx, 0);
             cudaError_t e = k3_launch(ctx, la, best, ctx->stream);

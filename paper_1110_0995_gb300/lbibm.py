@@ -376,7 +376,7 @@ class Simulation:
         return n.value, b.value
 
     def set_prefetch(self, nodes_ahead: int):
-        """L2 prefetch distance of the stream-collide kernel in lattice nodes (0: the library's own)."""
+        """L2 prefetch distance of the stream-collide kernel in lattice nodes (0: off)."""
         self._check(self._L.lb_set_prefetch(self._h, int(nodes_ahead)))
 
     def prefetch(self) -> int:

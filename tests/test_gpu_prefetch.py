@@ -1,0 +1,80 @@
+"""The stream-collide's L2 prefetch: off, the library's own distance where none
+was set, and set ones, on lattices that reach beyond them and on a batch; the
+autotuner's choice; and the backward walk of lattices about the size of L2."""
+import numpy as np
+import pytest
+
+from paper_1110_0995_gb300 import lbibm
+
+pytestmark = pytest.mark.gpu
+
+WIDE = (256, 64, 64)      # 1,048,576 nodes, beyond every distance below
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+
+    __graft_entry__.build()
+
+
+def _params(dims, storage, force=(1e-5, 3e-6, 0.0)):
+    return lbibm.make_params(dims, body_force=force, periodic=(1, 0, 0), storage=storage)
+
+
+def _fields(sim, steps=9):
+    sim.step(steps)
+    out = []
+    for k in range(len(sim.dims)):
+        sim.select(k)
+        out.append(np.concatenate([np.ravel(a) for a in sim.fields()]))
+    return np.concatenate(out)
+
+
+@pytest.mark.parametrize("storage,own", [("f32", 65536), ("f16", 131072), ("bf16", 131072)])
+def test_off_is_not_the_default(storage, own):
+    sim = lbibm.Simulation([_params(WIDE, storage)])
+    assert sim.prefetch() == own
+    sim.set_prefetch(0)
+    assert sim.prefetch() == 0
+    sim.set_prefetch(262144)
+    assert sim.prefetch() == 262144
+    small = lbibm.Simulation([_params((32, 16, 16), storage)])
+    assert small.prefetch() == 0
+
+
+@pytest.mark.parametrize("storage,variant", [("f32", (1, 128)), ("f32", (2, 128)), ("f16", (4, 64)), ("bf16", (2, 128))])
+@pytest.mark.parametrize("dims", [[WIDE], [(200, 48, 40), (64, 64, 64), (96, 40, 24)]])
+def test_results_do_not_depend_on_it(storage, variant, dims):
+    want = None
+    for d in (None, 0, 65536, 131072, 262144):
+        sim = lbibm.Simulation([_params(n, storage) for n in dims])
+        sim.set_kernel_config(*variant)
+        if d is not None:
+            sim.set_prefetch(d)
+        got = _fields(sim)
+        assert want is None or np.array_equal(got, want)
+        want = got
+
+
+def test_autotuner_reports_the_distance_in_use():
+    sim = lbibm.Simulation([_params(WIDE, "f32")])
+    npt, _, ms = sim.autotune(5)
+    assert ms > 0
+    if npt > 0:
+        assert sim.prefetch() in (0, 65536, 131072, 262144)
+    small = lbibm.Simulation([_params((64, 32, 16), "f32")])
+    if small.autotune(5)[0] > 0:
+        assert small.prefetch() == 0
+
+
+def test_backward_walk():
+    """110 MB of populations: odd steps walk the blocks backwards.  The same
+    channels in one context (220 MB) walk forwards only."""
+    dims, forces = (181, 75, 53), ((1e-5, 3e-6, 0.0), (2e-5, 0.0, 1e-6))
+    both = _fields(lbibm.Simulation([_params(dims, "f32", f) for f in forces]), 8).reshape(2, -1)
+    for k, f in enumerate(forces):
+        alone = _fields(lbibm.Simulation([_params(dims, "f32", f)]), 8)
+        # (FP32 rounding of two forms of one kernel; density 1, velocities below 1e-3)
+        assert np.abs(alone - both[k]).max() <= 1e-6
+        assert np.abs(alone - both[1 - k]).max() > 1e-5
