@@ -26,6 +26,7 @@ namespace {
 
 constexpr int CHUNK_TRIS = 128;     // triangles per block of the area/volume reduction (one per thread)
 constexpr int MAX_VALENCE = 64;
+constexpr int DIAG_OUT = 9;         // lb_diagnostics' sums and three error words
 
 struct ChannelHost {
     lb_params p;
@@ -105,8 +106,7 @@ struct lb_ctx {
     float4* u = nullptr;
     ChannelDev* d_ch = nullptr;
     char* diag_partials = nullptr;
-    double* diag_out = nullptr;      // [9], page-locked host memory that the kernel writes: the sums of
-                                     // lb_diagnostics and the error words
+    double* diag_own = nullptr;      // [DIAG_OUT] of a context without cells (see lb_diagnostics)
     unsigned* diag_done = nullptr;
     int diag_blocks = 0;
     // immersed boundary, host staging
@@ -842,7 +842,7 @@ void apply_k3_config(lb_ctx* ctx, K3Config c) {
 
 // The element tables of every mesh (triangles with their rest
 // areas, edges with rest length and rest dihedral angle (the bending's
-// theta0, Sec. 2.3.1)), written at the commit, the
+// theta0, Sec. 2.3.1)), then after(mesh), at the commit, the
 // meshes spread over up to 16 host threads (each writes only its own ranges).
 template <class After>
 void build_tables(lb_ctx* ctx, After after) {
@@ -902,7 +902,6 @@ lb_status commit_tables(lb_ctx* ctx) {
     // the patches of every distinct connectivity, then the cells' jobs on them
     PatchTables ptabs;
     std::vector<PatchJob> hpatches;
-    std::vector<int> cell_patch0(ctx->hcells.size(), 0);
     int n_rest[3] = {0, 0, 0};
     for (const PendingMesh& pm : ctx->pending_meshes) {
         MeshConn& c = *pm.conn;
@@ -925,23 +924,18 @@ lb_status commit_tables(lb_ctx* ctx) {
             append(ptabs.tri_id, t.tri_id);
             append(ptabs.edge_id, t.edge_id);
         }
-        // positions relative to the reference node split at 2^-grid: 16 where the
-        // cell reaches at most 64 lu from it, so that the upper parts (23 bits
-        // with room for twice the extent) and the lower ones are exact in FP32
-        const double* x = ctx->hrest.data() + 3 * (size_t)pm.node0;
-        double ext = 1.0;
-        for (int k = 0; k < 3 * c.n; ++k) ext = std::max(ext, std::fabs(x[k] - x[k % 3]));
         const CellDev& cd = ctx->hcells[pm.cell];
         PatchJob job = {};
         job.cell = pm.cell;
         job.ref = cd.ref;
         job.node0 = pm.node0;
-        job.grid = std::max(0, std::min(16, 22 - (int)std::ceil(std::log2(ext))));
-        job.patch0 = cell_patch0[pm.cell] = (int)hpatches.size();
+        job.patch0 = (int)hpatches.size();
         job.n_patch = c.n_patch;
         job.ks = cd.ks;
         job.kb = cd.kb;
         job.kal = cd.kal;
+        job.e0 = pm.e0;
+        job.tri0 = pm.tri0;
         for (int k = 0; k < c.n_patch; ++k) {
             job.tab = ptabs.tab[c.patch0 + k];
             job.rest_edge = n_rest[0];
@@ -955,26 +949,17 @@ lb_status commit_tables(lb_ctx* ctx) {
     }
     ctx->n_patches = (int)hpatches.size();
     for (const PatchTab& t : ptabs.tab) ctx->patch_smem = std::max(ctx->patch_smem, patch_smem_bytes(t));
-    std::vector<float2> rest_edge(n_rest[0]);
-    std::vector<float> rest_tri(n_rest[1]);
-    std::vector<Fix3> rest_node(n_rest[2]);
+    // positions relative to the reference node split at 2^-grid: 16 where the
+    // cell reaches at most 64 lu from it, so that the upper parts (23 bits
+    // with room for twice the extent) and the lower ones are exact in FP32
+    std::vector<int> grid(ctx->hcells.size(), 16);
     build_tables(ctx, [&](const PendingMesh& pm) {
-        // a cell's rest data in its patches' order
-        const CellDev& cd = ctx->hcells[pm.cell];
-        const Q4 r = ctx->hq0[cd.ref];
-        for (int b = cell_patch0[pm.cell], k = 0; k < pm.conn->n_patch; ++k, ++b) {
-            const PatchJob& j = hpatches[b];
-            for (int i = 0; i < j.tab.n_edge; ++i) {
-                const float4 e = ctx->hedge_rest[pm.e0 + ptabs.edge_id[j.tab.edge0 + i]];
-                rest_edge[j.rest_edge + i] = make_float2(e.x, e.y);
-            }
-            for (int i = 0; i < j.tab.n_tri; ++i) rest_tri[j.rest_tri + i] = ctx->htriS0[pm.tri0 + ptabs.tri_id[j.tab.tri0 + i]];
-            for (int i = 0; i < j.tab.n_loc; ++i) {
-                const Q4& q = ctx->hq0[pm.node0 + ptabs.loc[j.tab.loc0 + i]];
-                rest_node[j.rest_node + i] = Fix3{q.x - r.x, q.y - r.y, q.z - r.z};
-            }
-        }
+        const double* x = ctx->hrest.data() + 3 * (size_t)pm.node0;
+        double ext = 1.0;
+        for (int k = 0; k < 3 * pm.conn->n; ++k) ext = std::max(ext, std::fabs(x[k] - x[k % 3]));
+        grid[pm.cell] = std::max(0, std::min(16, 22 - (int)std::ceil(std::log2(ext))));
     });
+    for (PatchJob& j : hpatches) j.grid = grid[j.cell];
     ctx->M = (int)ctx->hq0.size();
     ctx->C = (int)ctx->hcells.size();
     ctx->T = (int)ctx->htris.size();
@@ -1030,17 +1015,44 @@ lb_status commit_tables(lb_ctx* ctx) {
     }
     LB_CUDA(up(&ctx->edges, ctx->hedges));
     LB_CUDA(up(&ctx->edge_rest, ctx->hedge_rest));
-    LB_CUDA(up(&ctx->patches, hpatches));
-    LB_CUDA(up(&ctx->ploc, ptabs.loc));
-    LB_CUDA(up(&ctx->ptri, ptabs.tri));
-    LB_CUDA(up(&ctx->pedge, ptabs.edge));
-    LB_CUDA(up(&ctx->pring, ptabs.ring));
-    LB_CUDA(up(&ctx->prest_edge, rest_edge));
-    LB_CUDA(up(&ctx->prest_tri, rest_tri));
-    LB_CUDA(up(&ctx->prest_node, rest_node));
+    // the patches' tables in one piece (most are small: an allocation and a copy
+    // of each took longer than its bytes)
+    std::vector<char> tabs;
+    auto place = [&tabs](const auto& v) {
+        const size_t at = (tabs.size() + 255) & ~(size_t)255, bytes = v.size() * sizeof(v[0]);
+        tabs.resize(at + bytes);
+        if (bytes) std::memcpy(tabs.data() + at, v.data(), bytes);
+        return at;
+    };
+    const size_t at_jobs = place(hpatches), at_loc = place(ptabs.loc), at_tri = place(ptabs.tri), at_edge = place(ptabs.edge),
+                 at_ring = place(ptabs.ring), at_tri_id = place(ptabs.tri_id), at_edge_id = place(ptabs.edge_id);
+    char* dtabs = nullptr;
+    LB_CUDA(up(&dtabs, tabs));
+    ctx->patches = (PatchJob*)(dtabs + at_jobs);
+    ctx->ploc = (uint32_t*)(dtabs + at_loc);
+    ctx->ptri = (uint2*)(dtabs + at_tri);
+    ctx->pedge = (uint2*)(dtabs + at_edge);
+    ctx->pring = (uint2*)(dtabs + at_ring);
     LB_CUDA(dalloc(ctx, &ctx->acc, 3 * (size_t)ctx->M));
     LB_CUDA(up(&ctx->tris, ctx->htris));
     LB_CUDA(up(&ctx->triS0, ctx->htriS0));
+    {
+        PatchRest r = {};
+        LB_CUDA(dalloc(ctx, &ctx->prest_edge, n_rest[0]));
+        LB_CUDA(dalloc(ctx, &ctx->prest_tri, n_rest[1]));
+        LB_CUDA(dalloc(ctx, &ctx->prest_node, n_rest[2]));
+        r.jobs = ctx->patches;
+        r.loc = ctx->ploc;
+        r.tri_id = (const int*)(dtabs + at_tri_id);
+        r.edge_id = (const int*)(dtabs + at_edge_id);
+        r.edge_rest = ctx->edge_rest;
+        r.tri_S0 = ctx->triS0;
+        r.q0 = ctx->q0;
+        r.rest_edge = ctx->prest_edge;
+        r.rest_tri = ctx->prest_tri;
+        r.rest_node = ctx->prest_node;
+        LB_CUDA(launch_patch_rest(r, ctx->n_patches, ctx->stream));
+    }
     LB_CUDA(up(&ctx->chunks, ctx->hchunks));
     LB_CUDA(up(&ctx->d_cells, ctx->hcells));
     LB_CUDA(dalloc(ctx, &ctx->F, ctx->M));
@@ -1048,7 +1060,8 @@ lb_status commit_tables(lb_ctx* ctx) {
         LB_CUDA(dalloc(ctx, &ctx->W, ctx->M));
         LB_CUDA(cudaMemsetAsync(ctx->W, 0, sizeof(float4) * ctx->M, ctx->stream));
     }
-    LB_CUDA(cudaMallocHost((void**)&ctx->hq_pinned, sizeof(Q4) * (size_t)ctx->M));
+    // (and the result of lb_diagnostics behind the positions)
+    LB_CUDA(cudaMallocHost((void**)&ctx->hq_pinned, sizeof(Q4) * (size_t)ctx->M + DIAG_OUT * sizeof(double)));
     LB_CUDA(cudaMemsetAsync(ctx->F, 0, sizeof(float4) * ctx->M, ctx->stream));
     LB_CUDA(dalloc(ctx, &ctx->partials, std::max(ctx->NCH, ctx->n_patches)));
     LB_CUDA(dalloc(ctx, &ctx->counters, ctx->C));
@@ -1237,7 +1250,6 @@ lb_status lb_create_batch(const lb_params* params, int n_channels, void* cuda_st
     TRY(dalloc(ctx, &ctx->d_ch, ctx->ch.size()));
     ctx->diag_blocks = ctx->sm_count * 4;
     TRY(dalloc(ctx, &ctx->diag_partials, diag_partial_bytes(ctx->diag_blocks)));
-    TRY(cudaMallocHost((void**)&ctx->diag_out, 9 * sizeof(double)));
     TRY(dalloc(ctx, &ctx->diag_done, 1));
     TRY(cudaMemsetAsync(ctx->diag_done, 0, sizeof(unsigned), ctx->stream));
     TRY(cudaMemsetAsync(ctx->h[0], 0, (size_t)Q * ctx->plane * pop_bytes(ctx->storage), ctx->stream));
@@ -1313,7 +1325,7 @@ lb_status lb_destroy(lb_ctx* ctx) {
     drop_graphs(ctx);
     for (void* p : ctx->allocations) cudaFree(p);
     if (ctx->hq_pinned) cudaFreeHost(ctx->hq_pinned);
-    if (ctx->diag_out) cudaFreeHost(ctx->diag_out);
+    if (ctx->diag_own) cudaFreeHost(ctx->diag_own);
     ctx->allocations.clear();
     for (auto& ep : ctx->pending) { cudaEventDestroy(ep.a); cudaEventDestroy(ep.b); }
     for (auto e : ctx->free_events) cudaEventDestroy(e);
@@ -2554,9 +2566,16 @@ lb_status lb_diagnostics(lb_ctx* ctx, double u_max, double out[6]) {
     LB_GUARD(ctx);
     if (!out) return LB_ERR_ARG;
     const ChannelHost& c = ctx->ch[ctx->cur];
-    const double* res = ctx->diag_out;
+    // page-locked host memory that the kernel writes: the sums and the error
+    // words, behind the staged positions, or a piece of its own when there are
+    // none (allocated by the first call: at creation it cost every context 0.15 ms)
+    double* res = ctx->hq_pinned ? (double*)(ctx->hq_pinned + ctx->M) : ctx->diag_own;
+    if (!res) {
+        LB_CUDA(cudaMallocHost((void**)&ctx->diag_own, DIAG_OUT * sizeof(double)));
+        res = ctx->diag_own;
+    }
     LB_CUDA(launch_diagnostics(lattice_args(ctx, (int)(ctx->step & 1)), ctx->cur, c.d.n, ctx->diag_partials,
-                               ctx->diag_blocks, ctx->diag_done, ctx->rep_err, ctx->sched_err, ctx->diag_out, ctx->stream));
+                               ctx->diag_blocks, ctx->diag_done, ctx->rep_err, ctx->sched_err, res, ctx->stream));
     LB_CUDA(cudaStreamSynchronize(ctx->stream));
     std::copy(res, res + 6, out);
     if (out[4] > 0) return fail(ctx, LB_ERR_NUMERIC, "non-finite populations");

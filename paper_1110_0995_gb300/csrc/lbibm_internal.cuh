@@ -172,7 +172,8 @@ struct __align__(16) PatchJob {
     int cell, ref, node0, grid, patch0, n_patch;   // of the cell
     int rest_edge, rest_tri, rest_node;            // offsets of its rest data
     float ks, kb, kal;
-    int pad[3];
+    int e0, tri0;                                  // its first edge and triangle in the context's tables
+    int pad;
 };
 struct Fix3 {
     long long x, y, z;
@@ -435,6 +436,19 @@ struct PatchTables {
 };
 void build_patches(const MeshTables& m, PatchTables& out);   // host
 size_t patch_smem_bytes(const PatchTab& t);
+// The patches' rest data (IbmArgs::prest_*) from the cells' tables.
+struct PatchRest {
+    const PatchJob* jobs;
+    const uint32_t* loc;
+    const int *tri_id, *edge_id;
+    const float4* edge_rest;
+    const float* tri_S0;
+    const Q4* q0;
+    float2* rest_edge;
+    float* rest_tri;
+    Fix3* rest_node;
+};
+cudaError_t launch_patch_rest(const PatchRest& r, int n_patches, cudaStream_t s);
 cudaError_t launch_membrane(const IbmArgs& a, cudaStream_t s);
 cudaError_t launch_forces_spread(const IbmArgs& a, cudaStream_t s);
 cudaError_t launch_gfix_to_g(const IbmArgs& a, cudaStream_t s);

@@ -378,6 +378,22 @@ __global__ void __launch_bounds__(MB, MINB) k_membrane(const __grid_constant__ I
     if (a.W) pdl_entry();
 }
 
+// Once, when the context commits: a block per patch.  (Gathered on the host, with
+// their upload, the rest data cost the 62-cell filter 0.4 ms of its first step.)
+__global__ void __launch_bounds__(MB) k_patch_rest(const PatchRest r) {
+    const PatchJob J = r.jobs[blockIdx.x];
+    for (int i = threadIdx.x; i < J.tab.n_edge; i += MB) {
+        const float4 e = r.edge_rest[J.e0 + r.edge_id[J.tab.edge0 + i]];
+        r.rest_edge[J.rest_edge + i] = make_float2(e.x, e.y);
+    }
+    for (int i = threadIdx.x; i < J.tab.n_tri; i += MB) r.rest_tri[J.rest_tri + i] = r.tri_S0[J.tri0 + r.tri_id[J.tab.tri0 + i]];
+    const Q4 ref = r.q0[J.ref];
+    for (int i = threadIdx.x; i < J.tab.n_loc; i += MB) {
+        const Q4 q = r.q0[J.node0 + (int)r.loc[J.tab.loc0 + i]];
+        r.rest_node[J.rest_node + i] = Fix3{q.x - ref.x, q.y - ref.y, q.z - ref.z};
+    }
+}
+
 // Shared memory of one patch.
 size_t patch_bytes(const PatchTab& t) {
     return 48 * (size_t)t.n_loc + 24 * (size_t)(t.n_edge + t.n_tri);
@@ -535,6 +551,12 @@ void build_patches(const MeshTables& m, PatchTables& out) {
 }
 
 size_t patch_smem_bytes(const PatchTab& t) { return patch_bytes(t); }
+
+cudaError_t launch_patch_rest(const PatchRest& r, int n_patches, cudaStream_t s) {
+    if (n_patches <= 0) return cudaSuccess;
+    k_patch_rest<<<n_patches, MB, 0, s>>>(r);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_membrane(const IbmArgs& a, cudaStream_t s) {
     if (a.n_patches <= 0) return cudaSuccess;
