@@ -46,6 +46,7 @@ static __device__ __align__(256) double2 g_noalloc_partials[NA_MAX_PARTIALS];
 std::mutex g_setup_mutex;
 void* g_scratch_ptr[NA_MAX_DEVICES] = {};
 unsigned long long g_scratch_ctx[NA_MAX_DEVICES] = {};
+int g_sms[NA_MAX_DEVICES] = {};
 
 // Unique id of the context current on the calling thread (driver entry points
 // through the runtime, so the library needs no link against libcuda).
@@ -72,10 +73,10 @@ cudaError_t current_context_id(unsigned long long* id) {
     return cudaSuccess;
 }
 
-// Device address of the scratch array in the current context, looked up
-// (under a lock) on the first call on a device and whenever that device's
-// current context has changed since the last lookup.
-cudaError_t scratch_address(double2** out) {
+// Device address of the scratch array in the current context and the device's
+// SM count, looked up (under a lock) on the first call on a device and whenever
+// that device's current context has changed since the last lookup.
+cudaError_t scratch_address(double2** out, int* sms) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -89,10 +90,13 @@ cudaError_t scratch_address(double2** out) {
         if (e != cudaSuccess) return e;
         e = current_context_id(&id);
         if (e != cudaSuccess) return e;
+        e = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
         g_scratch_ptr[dev] = p;
         g_scratch_ctx[dev] = id;
     }
     *out = (double2*)g_scratch_ptr[dev];
+    *sms = g_sms[dev];
     return cudaSuccess;
 }
 
@@ -244,11 +248,12 @@ extern "C" lb_status ibm_area_volume_noalloc(const double* xyz, const int32_t* t
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // looked up on either path: any call before a capture prepares every later one
     double2* scratch = nullptr;
-    if (scratch_address(&scratch) != cudaSuccess) return LB_ERR_CUDA;
+    int sms = 0;
+    if (scratch_address(&scratch, &sms) != cudaSuccess) return LB_ERR_CUDA;
     int max_tris = max_chunks * NA_BLOCK;
     if (max_tris <= NA_CLUSTER_TRIS) {
         int cluster = NA_CLUSTER;
-        while (cluster > 1 && (long long)cluster * n_cells > NA_RESIDENT * 152) cluster /= 2;
+        while (cluster > 1 && (long long)cluster * n_cells > (long long)NA_RESIDENT * sms) cluster /= 2;
         const double* x = xyz;
         const int *t = tris, *c0 = cell_tri_start;
         void* args[] = {(void*)&x, (void*)&t, (void*)&c0, (void*)&max_tris, (void*)&area, (void*)&volume};
