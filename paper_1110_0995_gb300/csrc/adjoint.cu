@@ -72,8 +72,6 @@ __device__ __forceinline__ void atomic_add3(float4* p, float x, float y, float z
     atomicAdd(p, make_float4(x, y, z, 0.f));   // one 16-byte vector reduction
 }
 
-__device__ __forceinline__ const ChannelDev& achan(const AdjArgs& a) { return a.ch; }
-
 // ---------------------------------------------------------------------------
 // trilinear stencil of a fixed-point position (same weights as the forward:
 // 24-bit fractions), with the gradient of each weight

@@ -15,10 +15,8 @@
 
 namespace lbibm {
 
-__device__ __forceinline__ float3 f3(const float4& v) { return make_float3(v.x, v.y, v.z); }
 __device__ __forceinline__ float3 operator+(float3 a, float3 b) { return make_float3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ float3 operator-(float3 a, float3 b) { return make_float3(a.x - b.x, a.y - b.y, a.z - b.z); }
-__device__ __forceinline__ float3 operator-(float3 a) { return make_float3(-a.x, -a.y, -a.z); }
 __device__ __forceinline__ float3 operator*(float s, float3 a) { return make_float3(s * a.x, s * a.y, s * a.z); }
 __device__ __forceinline__ float dot(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ float3 cross(float3 a, float3 b) {
@@ -125,7 +123,6 @@ __device__ __forceinline__ float tri_dV6(const Pt& R, const Pt& P0, const Pt& P1
 // and independent of their order, and run on the integer pipe: this GPU's
 // FP64 pipe retires about two operations per clock per SM).  The last block
 // of a cell adds the cell's partials and forms dS, dV in FP64 once.
-// ---------------------------------------------------------------------------
 // ---------------------------------------------------------------------------
 // Block size and register budget of the immersed-boundary kernels: 128
 // threads within 64 registers (8192 per block), so that one such block fits

@@ -379,17 +379,8 @@ __device__ __forceinline__ Mac macro_brinkman(const float h[Q], float gx, float 
 // BGK collision with Guo forcing on shifted populations:
 //   h*_i = h_i + omega (h_i^eq - h_i) + S_i,
 //   h_i^eq = w_i [drho + rho (3 e.u + 9/2 (e.u)^2 - 3/2 u.u)],
-//   S_i = (1 - 1/2tau) w_i [3 (e_i - u) + 9 (e_i.u) e_i] . g.
-template <int I>
-__device__ __forceinline__ float collide_one(float hi, const Mac& m, float omega, float fpre) {
-    const float eu = ex(I) * m.ux + ey(I) * m.uy + ez(I) * m.uz;
-    const float eg = ex(I) * m.gx + ey(I) * m.gy + ez(I) * m.gz;
-    const float heq = wgt(I) * (m.drho + m.rho * (3.0f * eu + 4.5f * eu * eu - 1.5f * m.uu));
-    const float s = fpre * wgt(I) * (3.0f * (eg - m.ug) + 9.0f * eu * eg);
-    return hi + omega * (heq - hi) + s;
-}
-
-// The same collision for the pair of opposite directions (I, I+1), I odd:
+//   S_i = (1 - 1/2tau) w_i [3 (e_i - u) + 9 (e_i.u) e_i] . g,
+// for the pair of opposite directions (I, I+1), I odd:
 // e_{I+1} = -e_I, so the equilibrium and the source split into a part even in
 // e (shared) and a part odd in e (sign flipped), which halves the arithmetic.
 template <int I>
@@ -471,7 +462,7 @@ __device__ __forceinline__ void bounce_back(const S* src, long long NT, int gi, 
 // registers); four: 256 (255 registers).  (256x128x64 on GB300: FP32 1280 61.0
 // us, 1152 60.6, 1024 64.1; 16-bit: 1280 56.2, 1152 55.9, 1024 58.3.)  The
 // WIDE form of the FP32 kernel, one channel with its constants in the parameter
-// bank, fits 1280 threads (48 registers) without spilling: 256x128x64 57.2
+// bank, fits 1280 threads (48 registers, two of them spilled): 256x128x64 57.2
 // against 58.0 us, 512x256x128 409 against 411-418, while lattices of a few
 // waves wait on each warp's latency, which the smaller budget lengthens
 // (96x48x32 reproducible cycle 18.8 -> 19.1 us, 128x64x64 differentiable 1 %),
@@ -1061,10 +1052,12 @@ __global__ void __launch_bounds__(BS, LBIBM_K3_PAIR_THREADS / BS) k_stream_colli
 // are collided one after the other, each unpacked twice (for the moments and,
 // two directions at a time, for the collision), and the rounded results take
 // the words' place until each direction leaves as one 64-bit store.  That
-// fits 96 registers, 20 warps per SM; with a pair's 19 directions held as
-// floats it took 128, 16 warps, and stored 32-bit words.  Measured on GB300,
-// 512x256x128 FP16: 345 -> 315 us (two unpackings and 64-bit stores at 16
-// warps), 289 (20 warps), 261 (read-only loads); 24 warps spill, 282.
+// runs in 96 registers, 20 warps per SM, with 272 bytes a thread spilled and
+// 212 read back, which cost less than the four warps more give; with a pair's
+// 19 directions held as floats it took 128 registers, 16 warps, and stored
+// 32-bit words.  Measured on GB300, 512x256x128 FP16: 345 -> 315 us (two
+// unpackings and 64-bit stores at 16 warps), 289 (20 warps), 261 (read-only
+// loads); at 24 warps more is spilled, 282.
 // ---------------------------------------------------------------------------
 template <class S> struct QuadIO;
 template <> struct QuadIO<__half> {

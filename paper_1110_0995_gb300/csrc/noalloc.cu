@@ -122,7 +122,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // chunks of 256 keep the two launches, which spread one cell over any number of SMs.
 constexpr int NA_CLUSTER = 8;
 constexpr int NA_CLUSTER_TRIS = 32 * NA_BLOCK;
-constexpr int NA_RESIDENT = 6;                // blocks per SM at 40 registers a thread
+constexpr int NA_RESIDENT = 6;                // blocks per SM at 40 registers a thread (24 bytes spilled)
 
 // (area x 2, volume x 6) of triangle t, added to s and v.
 __device__ __forceinline__ void triangle_terms(const double* __restrict__ xyz, const int* __restrict__ tris, int t,
