@@ -251,8 +251,9 @@ lb_status lb_get_kernel_config(lb_ctx* ctx, int* nodes_per_thread, int* block_si
  * 256 up to 2^24, else LB_ERR_ARG.  The bound on the useful distance is the L2
  * (19 x 4 bytes per node of distance for FP32 storage).  A context for which
  * none was set uses the library's own distance, five megabytes of populations
- * (65,536 nodes in FP32, 131,072 in 16 bits; off on lattices with fewer).
- * lb_get_prefetch: the distance in use. */
+ * (65,536 nodes in FP32, 131,072 in 16 bits; off on lattices with fewer, and
+ * where L2 holds the populations: both buffers below 98 MiB in FP32, below
+ * 48 MiB in 16 bits).  lb_get_prefetch: the distance in use. */
 lb_status lb_set_prefetch(lb_ctx* ctx, int nodes_ahead);
 lb_status lb_get_prefetch(lb_ctx* ctx, int* nodes_ahead);
 

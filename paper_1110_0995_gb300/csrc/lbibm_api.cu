@@ -323,25 +323,41 @@ __global__ void k_guard_count(const unsigned char* __restrict__ p, size_t n, uns
 
 size_t pop_bytes(lb_storage s) { return s == LB_F32 ? 4 : 2; }
 
+// The size of the two population buffers against L2 (126 MB) decides two rules
+// below.  Cycles on GB300, us, filters with cells (channels without in brackets),
+// by MiB of both buffers:
+//   FP32, prefetch off / on, forwards:  21 15.08 / 15.42, 76 23.53 / 24.44,
+//     95 29.67 / 29.74 (18.21 / 19.14), 103 32.44 / 32.34, 142 41.7 / 40.0
+//   with it, forwards / backwards:  76 24.44 / 24.62, 95 29.74 / 29.83,
+//     100 31.39 / 30.81, 120 36.2 / 34.6, 180 46.7 / 45.7 (228 38.5 / 38.0)
+//   BF16, prefetch off / on, forwards:  38 22.21 / 22.26 (43 11.63 / 11.70),
+//     59 27.70 / 27.34 (14.78 / 15.08), 89 39.3 / 38.1, 180 63.9 / 59.7
+//   with it, forwards / backwards:  59 27.34 / 27.68, 89 38.1 / 36.4, 180 59.7 / 58.7
+// Populations that L2 holds gain nothing from being asked for early and pay for
+// the request: off below 98 MiB in FP32, and below 48 in 16 bits, whose kernel
+// waits longer on L2.
+size_t population_bytes(const lb_ctx* ctx) { return 2 * (size_t)Q * ctx->plane * pop_bytes(ctx->storage); }
+size_t prefetch_min(const lb_ctx* ctx) { return (size_t)(ctx->storage == LB_F32 ? 98 : 48) << 20; }
+
 // The stream-collide's L2 prefetch distance where none was set: five
 // megabytes of populations, 65,536 nodes in FP32 and 131,072 in 16 bits, about
 // what the resident blocks hold in flight (GB300, without / with: 256x128x64
 // FP32 60.0 / 57.2 us, 512x256x128 FP32 411 / 409, FP16 261 / 246; half the
 // distance 1-4 us slower, twice no faster).
 constexpr int PREFETCH_BYTES = Q * 65536 * 4;
-// The distance in use: the set one, or the library's own, 0 where the lattice
-// has no node that far ahead.
+// The distance in use: the set one, or the library's own, 0 below prefetch_min
+// and where the lattice has no node that far ahead.
 int prefetch_nodes(const lb_ctx* ctx) {
     if (ctx->pf_nodes >= 0) return ctx->pf_nodes;
     const int d = PREFETCH_BYTES / (Q * (int)pop_bytes(ctx->storage));
-    return d < ctx->Ntot ? d : 0;
+    return d < ctx->Ntot && population_bytes(ctx) >= prefetch_min(ctx) ? d : 0;
 }
 // Odd steps walk the blocks backwards when both population buffers together
-// are about the size of L2 (126 MB, three quarters to three halves): they then
-// begin with what the previous step wrote last.  Measured on GB300: 181x75x53
-// FP32, 110 MB, 36.3 -> 35.3 us per cycle; 256x128x64 FP32, 319 MB, 70.4 ->
-// 71.2; populations that stay in L2 anyway lose the die they lie on (32x16x64,
-// 5 MB: 11.7 -> 12.7; 128x64x64 differentiable, 80 MB, 1 % slower).
+// are about the size of L2 (three quarters, FP32 from where the prefetch begins,
+// to three halves): they then begin with what the previous step wrote last.
+// Beyond, the gain fades (256x128x64 FP32 with cells, 304 MiB, 70.4 -> 71.2 us
+// per cycle); populations that stay in L2 anyway lose the die they lie on
+// (32x16x64, 5 MB: 11.7 -> 12.7; 128x64x64 differentiable, 76 MiB, 1 % slower).
 constexpr size_t ZIGZAG_MIN = (size_t)94 << 20, ZIGZAG_MAX = (size_t)189 << 20;
 
 LatticeArgs lattice_args(const lb_ctx* ctx, int par) {
@@ -373,8 +389,8 @@ LatticeArgs lattice_args(const lb_ctx* ctx, int par) {
     a.tma_err = ctx->sched_err ? ctx->sched_err + 1 : nullptr;
     a.pf_nodes = prefetch_nodes(ctx);
     if (a.pf_nodes >= ctx->Ntot) a.pf_nodes = 0;   // nothing that far ahead
-    const size_t pops = 2 * (size_t)Q * ctx->plane * pop_bytes(ctx->storage);
-    a.rev = par && !ctx->phi && pops >= ZIGZAG_MIN && pops <= ZIGZAG_MAX;
+    const size_t pops = population_bytes(ctx);
+    a.rev = par && !ctx->phi && pops >= std::max(ZIGZAG_MIN, prefetch_min(ctx)) && pops <= ZIGZAG_MAX;
     return a;
 }
 

@@ -43,6 +43,16 @@ def test_off_is_not_the_default(storage, own):
     assert small.prefetch() == 0
 
 
+@pytest.mark.parametrize("storage,dims,own", [
+    ("f32", [(128, 64, 50)], 0), ("f32", [(160, 64, 60)], 0), ("f32", [(192, 72, 60)], 65536),
+    ("f32", [(96, 64, 48), (96, 64, 40)], 0), ("f32", [(96, 64, 80), (96, 64, 60)], 65536),
+    ("f16", [(128, 64, 64)], 0), ("f16", [(160, 64, 120)], 131072), ("bf16", [(96, 64, 96)], 0),
+])
+def test_off_where_l2_holds_the_populations(storage, dims, own):
+    """Asked for early, populations that are in L2 anyway cost up to 4 % of a cycle."""
+    assert lbibm.Simulation([_params(d, storage) for d in dims]).prefetch() == own
+
+
 @pytest.mark.parametrize("storage,variant", [("f32", (1, 128)), ("f32", (2, 128)), ("f16", (4, 64)), ("bf16", (2, 128))])
 @pytest.mark.parametrize("dims", [[WIDE], [(200, 48, 40), (64, 64, 64), (96, 40, 24)]])
 def test_results_do_not_depend_on_it(storage, variant, dims):
