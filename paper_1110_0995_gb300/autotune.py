@@ -18,7 +18,9 @@ def cache_path() -> str:
 
 
 def _key(device: str, storage: str, dims) -> str:
-    return f"{device}|{storage}|" + ";".join("x".join(str(v) for v in d) for d in dims)
+    # "2": what the entries mean (in earlier ones a distance of 0 stood for the
+    # library's own, so they are not read)
+    return f"2|{device}|{storage}|" + ";".join("x".join(str(v) for v in d) for d in dims)
 
 
 def _load() -> dict:

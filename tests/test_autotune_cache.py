@@ -59,3 +59,14 @@ def test_unwritable_cache_still_tunes(tmp_path, monkeypatch):
     s = FakeSim([(64, 32, 32)])
     r = autotune.tune(s, "GB300", "f32")
     assert not r["cached"] and s.timed == 1
+
+
+def test_entries_of_another_meaning_are_not_used(tmp_path, monkeypatch):
+    """Entries without the key's version have a distance of 0 where the
+    prefetch was on: the variant is timed again."""
+    path = tmp_path / "at.json"
+    path.write_text('{"GB300|f32|64x32x32": {"npt": 4, "bs": 64, "pf": 0, "ms": 0.1}}')
+    monkeypatch.setenv("LBIBM_CACHE", str(path))
+    s = FakeSim([(64, 32, 32)])
+    r = autotune.tune(s, "GB300", "f32")
+    assert not r["cached"] and s.timed == 1 and s.config == (2, 256)
