@@ -282,8 +282,10 @@ lb_status lb_get_schedule(lb_ctx* ctx, int* overlapped);
 /* Autotuner: times every supported stream-collide variant on this context's
  * lattice (`repeats` launches each, CUDA events), selects the fastest, then
  * times its L2 prefetch distances (off, 65536, 131072, 262144 nodes, as far as
- * the lattice reaches; variants with 1, 2 or 4 nodes per thread) and keeps the fastest (lb_get_prefetch
- * reads it), and returns the variant with its mean time per launch in ms.
+ * the lattice reaches; variants with 1, 2 or 4 nodes per thread) and keeps
+ * the library's own unless another is at least 1 % faster
+ * (lb_get_prefetch reads it), and returns the variant with its mean time per
+ * launch in ms.
  * Only before the first lb_step (LB_ERR_STATE otherwise): there, repeated
  * launches leave the state unchanged. */
 lb_status lb_autotune(lb_ctx* ctx, int repeats, int* nodes_per_thread, int* block_size, double* ms);

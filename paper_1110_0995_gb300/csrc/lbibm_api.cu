@@ -2267,17 +2267,22 @@ lb_status lb_autotune(lb_ctx* ctx, int repeats, int* nodes_per_thread, int* bloc
         }
     }
     // then the L2 prefetch distance of the winner (variants with 1, 2 or 4
-    // nodes per thread): off and the distances that the lattice reaches; the
-    // one kept is the fastest, the shorter on a tie
+    // nodes per thread): the library's own stays unless off or another distance
+    // that the lattice reaches is at least 1 % faster (launches alone, back to
+    // back, tell less than a cycle: 512x256x128 FP32 off and on within 1 %, in
+    // the cycle 477 and 471 us)
     apply_k3_config(ctx, best);
     if (ctx->ch.size() > (size_t)MAXCH_P && upload_channels(ctx) != LB_OK) return LB_ERR_CUDA;
     const int keep_pf = ctx->pf_nodes;
     int best_pf = keep_pf;
     if (best.npt > 0) {
-        const int dists[] = {0, 65536, 131072, 262144};
+        ctx->pf_nodes = -1;
+        const int own = prefetch_nodes(ctx);
+        const int dists[] = {own, 0, 65536, 131072, 262144};
         double best_pf_ms = 1e30;
-        for (int d : dists) {
-            if (d >= ctx->Ntot) continue;
+        for (int k = 0; k < 5; ++k) {
+            const int d = dists[k];
+            if (d >= ctx->Ntot || (k > 0 && d == own)) continue;
             ctx->pf_nodes = d;
             const LatticeArgs la = lattice_args(ctx, 0);
             cudaError_t e = k3_launch(ctx, la, best, ctx->stream);

@@ -88,3 +88,14 @@ def test_backward_walk():
         # (FP32 rounding of two forms of one kernel; density 1, velocities below 1e-3)
         assert np.abs(alone - both[k]).max() <= 1e-6
         assert np.abs(alone - both[1 - k]).max() > 1e-5
+
+
+def test_autotuner_keeps_the_own_distance_on_a_tie():
+    """Timed alone, the large filter's launches are within 1 % with the prefetch
+    off and on; in a cycle on is 1.3 % faster, so off has to win clearly."""
+    from paper_1110_0995_gb300 import scene
+
+    sc = scene.micropost_filter(seed=31, dims=(512, 256, 128), cols=8, rows=4, n_rbc=0, n_ctc=0)
+    sim = lbibm.Simulation.from_scenes([sc], "f32")
+    assert sim.autotune(20)[0] > 0
+    assert sim.prefetch() > 0
